@@ -114,7 +114,7 @@ FSMP_HD void philox4x64_10(uint64_t c[4], uint64_t k0, uint64_t k1) {
   const uint64_t M0 = 0xD2E7470EE14C6C93ULL, M1 = 0xCA5A826395121157ULL;
   const uint64_t W0 = 0x9E3779B97F4A7C15ULL, W1 = 0xBB67AE8584CAA73BULL;
 #ifdef __CUDA_ARCH__
-#pragma unroll
+#pragma unroll 1
 #endif
   for (int r = 0; r < 10; ++r) {
     if (r > 0) { k0 += W0; k1 += W1; }
@@ -152,19 +152,24 @@ template <typename F, int L>
 __device__ inline F lmle_newton(const int* h, int bot, int top, F lambda0, F lam, F& lo, F& hi, F tol, int max_it,
                                 int sl, unsigned gm, F* ll_out) {
   F ll = -INFINITY;
+#pragma unroll 1
   for (int it = 0; it < max_it; ++it) {
     if (hi - lo <= tol * hi) break;  // the bracket has closed
     const F s = log(lam / lambda0);
     F mx = -INFINITY;
+#pragma unroll 1
     for (int k = bot + sl; k <= top; k += L)
       if (h[k] > 0) mx = fmax(mx, log((F)h[k]) + k * s);
+#pragma unroll 1
     for (int o = L / 2; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(gm, mx, o, L));
     F sw = 0, s1 = 0, s2 = 0;
+#pragma unroll 1
     for (int k = bot + sl; k <= top; k += L)
       if (h[k] > 0) {
         const F e = exp(log((F)h[k]) + k * s - mx);
         sw += e; s1 += k * e; s2 += (F)k * k * e;
       }
+#pragma unroll 1
     for (int o = L / 2; o > 0; o >>= 1) {
       sw += __shfl_xor_sync(gm, sw, o, L);
       s1 += __shfl_xor_sync(gm, s1, o, L);
@@ -188,8 +193,10 @@ __device__ inline F lmle_newton(const int* h, int bot, int top, F lambda0, F lam
 template <int L>
 __device__ inline double group_lambda_mle(const int* h, int n_max, double lambda0, int sl, unsigned gm) {
   int top = -1, bot = n_max + 1;
+#pragma unroll 1
   for (int k = sl; k <= n_max; k += L)
     if (h[k] > 0) { top = k; bot = min(bot, k); }
+#pragma unroll 1
   for (int o = L / 2; o > 0; o >>= 1) {
     top = max(top, __shfl_xor_sync(gm, top, o, L));
     bot = min(bot, __shfl_xor_sync(gm, bot, o, L));
@@ -202,18 +209,22 @@ __device__ inline double group_lambda_mle(const int* h, int n_max, double lambda
   const float lr0 = log2f((float)lambda0);
   float best = -INFINITY;
   int bi = 0;
+#pragma unroll 1
   for (int g = sl; g < G; g += L) {
     const float lam = (float)top * (float)(g + 1) / (float)G;
     const float s2 = log2f(lam) - lr0;
     float mx = -INFINITY;
+#pragma unroll 1
     for (int k = bot; k <= top; ++k)
       if (h[k] > 0) mx = fmaxf(mx, log2f((float)h[k]) + (float)k * s2);
     float acc = 0.0f;
+#pragma unroll 1
     for (int k = bot; k <= top; ++k)
       if (h[k] > 0) acc += exp2f(log2f((float)h[k]) + (float)k * s2 - mx);
     const float l = -lam * 1.44269504f + mx + log2f(acc);
     if (l > best) { best = l; bi = g; }
   }
+#pragma unroll 1
   for (int o = L / 2; o > 0; o >>= 1) {  // argmax, the smaller index on ties
     const float ob = __shfl_xor_sync(gm, best, o, L);
     const int oi = __shfl_xor_sync(gm, bi, o, L);
@@ -270,6 +281,7 @@ cudaError_t measure_peaks(int sm_count, double* smem_gbs, double* fp64_tflops, d
 // workspace doubles per chain slot (FP32 mode); entries of a global C^-1 slot; ints of an N
 // histogram slot.
 size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns);
+size_t pe_limit_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns);
 size_t pe_ws_slot_doubles(int n_cap);
 size_t pe_c_entries(int n_cap);  // entries of a global C^-1 slot (packed triangle)
 size_t pe_c_entry_bytes(int precision);  // bytes of one C^-1 entry (a pair of FP64 or FP32 values)

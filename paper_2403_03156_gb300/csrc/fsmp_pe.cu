@@ -1,19 +1,40 @@
 // fsmp_pe.cu -- host side of the PE-space chain kernel (arXiv 2403.03156, Sec. 2.4 and Appendix
 // A.1) and its dynode-model instances; the kernel itself is in fsmp_pe_kernel.cuh.
+#include <type_traits>
+
 #include "fsmp_pe_kernel.cuh"
 
 namespace fsmp {
 
 size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns) {
   const int chains = warps * (32 / lanes);
-  const bool l16 = lanes == 16;
-  if (M.precision == FSMP_FP64)
-    return pe_block_bytes<double>(M) +
-           (size_t)chains * (l16 ? pe_chain_bytes<double, 16>(M.n_cap, n_alloc, M.win_extra, Ns)
-                                 : pe_chain_bytes<double, 32>(M.n_cap, n_alloc, M.win_extra, Ns));
-  return pe_block_bytes<float>(M) +
-         (size_t)chains * (l16 ? pe_chain_bytes<float, 16>(M.n_cap, n_alloc, M.win_extra, Ns)
-                               : pe_chain_bytes<float, 32>(M.n_cap, n_alloc, M.win_extra, Ns));
+  auto bytes = [&](auto big, auto lane_count, auto mix) {
+    constexpr bool BIG = decltype(big)::value, MIX = decltype(mix)::value;
+    constexpr int L = decltype(lane_count)::value;
+    if (M.precision == FSMP_FP64)
+      return pe_block_bytes<double>(M) + chains * pe_chain_bytes<double, BIG, L, MIX>(M.n_cap, n_alloc, M.win_extra, Ns);
+    return pe_block_bytes<float>(M) + chains * pe_chain_bytes<float, BIG, L, MIX>(M.n_cap, n_alloc, M.win_extra, Ns);
+  };
+  using std::false_type;
+  using std::true_type;
+  const std::integral_constant<int, 16> l16;
+  const std::integral_constant<int, 32> l32;
+  if (M.n_comp > 1)
+    return lanes == 16 ? bytes(false_type{}, l16, true_type{}) : bytes(false_type{}, l32, true_type{});
+  if (pe_big(M.n_cap)) return bytes(true_type{}, l32, false_type{});
+  return lanes == 16 ? bytes(false_type{}, l16, false_type{}) : bytes(false_type{}, l32, false_type{});
+}
+
+// The state that sets how long a window and how large a capacity a context takes: per chain 216
+// bytes of sums, the draws of `lanes` steps, the lists and four vectors of n_cap PEs, the residual,
+// log Phi and the C^-1 tile; per CTA the SER, log(i) and 1 / i. It stays what it is when the
+// kernel's own layout changes, so that what is refused does not depend on the launch shape.
+size_t pe_limit_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns) {
+  const bool f64 = M.precision == FSMP_FP64;
+  const size_t ts = f64 ? 8 : 4, cs = 2 * ts, n_cap = (size_t)M.n_cap;
+  const size_t chain = a16(216) + a16((f64 ? 56 : 28) * (size_t)lanes) + 2 * a16(4 * n_cap) + a16(n_cap) +
+                       4 * a16(cs * n_cap) + a16(ts * n_alloc) + a16(ts * M.win_extra) + a16(cs * (size_t)tri(Ns));
+  return a16(ts * M.Lt) + a16(ts * (n_cap + 2)) + a16(8 * (n_cap + 2)) + (size_t)(warps * (32 / lanes)) * chain;
 }
 
 size_t pe_ws_slot_doubles(int n_cap) { return pe_ws_doubles(n_cap); }

@@ -26,7 +26,8 @@
 //
 // Layout: a chain runs on a group of L consecutive lanes (L = 32: a warp; L = 16: two chains per
 // warp, for chains with few PEs, where most of a step is work that every lane repeats); a CTA
-// holds several independent chains and a group takes chains from a launch-wide counter. C^-1 sits
+// holds several independent chains and a group takes chains from a launch-wide counter. A chain of
+// up to 32 PEs scores four steps at once (kSpec below). C^-1 sits
 // in a per-chain shared-memory tile (the packed triangle of Ns PEs) while N <= Ns and moves to the
 // chain's global slot (n_cap PEs) when a birth would exceed the tile. The counts of N after
 // burn-in (for lambda_FSMP) sit in a global slot per chain.
@@ -52,6 +53,15 @@ namespace fsmp {
 namespace {
 
 constexpr int kPeMaxThreads = 128;  // warps per CTA: at most 4
+constexpr int kSub = 4;  // subgroups of a chain's lanes that score a step each (see kSpec)
+
+// x, unknown to the compiler: keeps it from cloning a loop per value of a flag that is the same in
+// all of its passes (the clones tripled the accept's code, and code size is what binds here).
+__device__ __forceinline__ bool opaque(bool x) {
+  int v = x;
+  asm volatile("" : "+r"(v));
+  return v != 0;
+}
 
 // The lanes of one chain: L consecutive lanes of a warp. Exchanges and reductions stay inside the
 // group; gm is its lane mask. A step draws the random numbers of the next L steps (one per lane).
@@ -60,13 +70,20 @@ template <int L> struct Lanes {
   int g;        // group within the warp
   unsigned gm;  // lane mask of the group
 };
+template <> struct Lanes<32> {  // a whole warp: the mask is a constant, which its shuffles need no code for
+  int sl;
+  static constexpr int g = 0;
+  static constexpr unsigned gm = 0xffffffffu;
+};
 template <int L> __device__ __forceinline__ Lanes<L> pe_lanes() {
   static_assert(L == 32 || L == 16, "a chain runs on 32 or 16 lanes");
   const int lane = threadIdx.x & 31;
   Lanes<L> r;
   r.sl = lane & (L - 1);
-  r.g = lane / L;
-  r.gm = L == 32 ? 0xffffffffu : (((1u << L) - 1u) << (r.g * L));
+  if constexpr (L != 32) {
+    r.g = lane / L;
+    r.gm = ((1u << L) - 1u) << (r.g * L);
+  }
   return r;
 }
 // the group's lanes with p set, as bits 0 .. L-1
@@ -185,6 +202,80 @@ template <int L> __device__ __forceinline__ ff cshfl_xor(ff a, int o, unsigned g
 template <int L> __device__ __forceinline__ ff cshfl(ff a, int src, unsigned gm) {
   return ff{__shfl_sync(gm, a.hi, src, L), __shfl_sync(gm, a.lo, src, L)};
 }
+// Two state values side by side. The float-float operations run on both at once with this part's
+// packed FP32 instructions (one instruction for two lanes' worth of the same rounding): half the
+// instructions of the loops over C^-1, which wait on instruction supply. Every half rounds as the
+// single operation does.
+template <typename C> struct Pk;
+template <> struct Pk<dd> {
+  dd a, b;
+};
+template <> struct Pk<ff> {
+  unsigned long long hi, lo;  // (hi of the first, hi of the second), the same of lo
+};
+__device__ __forceinline__ unsigned long long f2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float f2_first(unsigned long long p) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+  return a;
+}
+__device__ __forceinline__ float f2_second(unsigned long long p) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+  return b;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// a - b, as b (-1) + a: the product is exact, so one rounding
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+  return f2_fma(b, 0xbf800000bf800000ull, a);
+}
+__device__ __forceinline__ Pk<dd> pk2(dd a, dd b) { return Pk<dd>{a, b}; }
+__device__ __forceinline__ Pk<ff> pk2(ff a, ff b) { return Pk<ff>{f2(a.hi, b.hi), f2(a.lo, b.lo)}; }
+__device__ __forceinline__ dd pk_first(Pk<dd> x) { return x.a; }
+__device__ __forceinline__ dd pk_second(Pk<dd> x) { return x.b; }
+__device__ __forceinline__ ff pk_first(Pk<ff> x) { return ff{f2_first(x.hi), f2_first(x.lo)}; }
+__device__ __forceinline__ ff pk_second(Pk<ff> x) { return ff{f2_second(x.hi), f2_second(x.lo)}; }
+__device__ __forceinline__ Pk<dd> pk_add(Pk<dd> x, Pk<dd> y) { return Pk<dd>{cadd(x.a, y.a), cadd(x.b, y.b)}; }
+__device__ __forceinline__ Pk<dd> pk_mul(Pk<dd> x, Pk<dd> y) { return Pk<dd>{cmul(x.a, y.a), cmul(x.b, y.b)}; }
+__device__ __forceinline__ Pk<ff> pk_quick(unsigned long long a, unsigned long long b) {
+  const unsigned long long s = f2_add(a, b);
+  return Pk<ff>{s, f2_sub(b, f2_sub(s, a))};
+}
+__device__ __forceinline__ Pk<ff> pk_add(Pk<ff> x, Pk<ff> y) {  // ff_add on both
+  const unsigned long long s = f2_add(x.hi, y.hi);
+  const unsigned long long bb = f2_sub(s, x.hi);
+  const unsigned long long e = f2_add(f2_sub(x.hi, f2_sub(s, bb)), f2_sub(y.hi, bb));
+  return pk_quick(s, f2_add(e, f2_add(x.lo, y.lo)));
+}
+__device__ __forceinline__ Pk<ff> pk_mul(Pk<ff> x, Pk<ff> y) {  // ff_mul on both
+  const unsigned long long p = f2_mul(x.hi, y.hi);
+  unsigned long long e = f2_fma(x.hi, y.hi, f2_mul(p, 0xbf800000bf800000ull));
+  e = f2_fma(x.hi, y.lo, e);
+  e = f2_fma(x.lo, y.hi, e);
+  return pk_quick(p, e);
+}
+template <typename C> __device__ __forceinline__ Pk<C> pk_fma(Pk<C> x, Pk<C> y, Pk<C> z) {
+  return pk_add(pk_mul(x, y), z);
+}
+
 // a scoring-precision value (T) as a state value
 __device__ __forceinline__ ff cfromf(float a) { return ff{a, 0.0f}; }
 __device__ __forceinline__ dd cfromf(double a) { return dd{a, 0.0}; }
@@ -233,21 +324,17 @@ template <> struct CmT<double> {
 // probability exceeds the uniform u, else the last component with G > 0. The comparison is
 // in FP64 in both modes, so the draw is the same as the FP64 reference's.
 __device__ __forceinline__ int pe_draw_comp(const DevModel& M, double u) {
+#pragma unroll 1
   for (int e = 0; e < M.n_comp; ++e)
     if (M.cm_cum[e] > u) return e;
   return M.cm_last;
 }
 
-// group sums of state values: over all lanes, or over lanes [0, m) (zero beyond m)
+// group sum of a state value
 template <int L, typename C> __device__ __forceinline__ C csum(C v, const Lanes<L> ln) {
 #pragma unroll 1
   for (int o = L / 2; o > 0; o >>= 1) v = cadd(v, cshfl_xor<L>(v, o, ln.gm));
   return v;
-}
-template <int L, typename C> __device__ __forceinline__ C csum_first(C v, int m, const Lanes<L> ln) {
-  for (int o = L / 2; o > 0; o >>= 1)
-    if (o < m) v = cadd(v, cshfl_xor<L>(v, o, ln.gm));
-  return cshfl<L>(v, 0, ln.gm);
 }
 
 // twice a state value (exact)
@@ -255,29 +342,46 @@ __device__ __forceinline__ double ctwice(double a) { return 2.0 * a; }
 __device__ __forceinline__ dd ctwice(dd a) { return dd{2.0 * a.hi, 2.0 * a.lo}; }
 __device__ __forceinline__ ff ctwice(ff a) { return ff{2.0f * a.hi, 2.0f * a.lo}; }
 
-// two group sums of state values in one butterfly
-template <int L, typename C> __device__ __forceinline__ void csum2(C& a, C& b, const Lanes<L> ln) {
+// The first offset of a butterfly over values that are zero on lanes >= m (m >= 0): the levels
+// above it would add zeros only, which leaves a normalised pair as it is.
+template <int L> __device__ __forceinline__ int first_level(int m) {
+  return m > L / 2 ? L / 2 : (m > 1 ? 1 << (31 - __clz(m - 1)) : 0);
+}
+// one or two group sums of state values that are zero on lanes >= m, the result on every lane
+template <int L, typename C> __device__ __forceinline__ C csum_m(C v, int m, const Lanes<L> ln) {
 #pragma unroll 1
-  for (int o = L / 2; o > 0; o >>= 1) {
-    const C a2 = cshfl_xor<L>(a, o, ln.gm), b2 = cshfl_xor<L>(b, o, ln.gm);
-    a = cadd(a, a2);
-    b = cadd(b, b2);
+  for (int o = first_level<L>(m); o > 0; o >>= 1) v = cadd(v, cshfl_xor<L>(v, o, ln.gm));
+  return m > L / 2 ? v : cshfl<L>(v, 0, ln.gm);
+}
+template <int L, typename C> __device__ __forceinline__ void csum2_m(C& a, C& b, int m, const Lanes<L> ln) {
+  Pk<C> p = pk2(a, b);
+#pragma unroll 1
+  for (int o = first_level<L>(m); o > 0; o >>= 1)
+    p = pk_add(p, pk2(cshfl_xor<L>(pk_first(p), o, ln.gm), cshfl_xor<L>(pk_second(p), o, ln.gm)));
+  a = pk_first(p);
+  b = pk_second(p);
+  if (m <= L / 2) {
+    a = cshfl<L>(a, 0, ln.gm);
+    b = cshfl<L>(b, 0, ln.gm);
   }
 }
 
 // four group sums in one butterfly (two state values, two scoring-precision values), so that
 // their shuffles and additions overlap
-template <int L, typename C, typename T>
+// (over the group's L lanes, or within its subgroups of GW lanes)
+template <int L, int GW, typename C, typename T>
 __device__ __forceinline__ void gsum4(C& a, C& b, T& x, T& y, const Lanes<L> ln) {
+  Pk<C> p = pk2(a, b);
 #pragma unroll 1
-  for (int o = L / 2; o > 0; o >>= 1) {
-    const C a2 = cshfl_xor<L>(a, o, ln.gm), b2 = cshfl_xor<L>(b, o, ln.gm);
+  for (int o = GW / 2; o > 0; o >>= 1) {
+    const C a2 = cshfl_xor<L>(pk_first(p), o, ln.gm), b2 = cshfl_xor<L>(pk_second(p), o, ln.gm);
     const T x2 = __shfl_xor_sync(ln.gm, x, o, L), y2 = __shfl_xor_sync(ln.gm, y, o, L);
-    a = cadd(a, a2);
-    b = cadd(b, b2);
+    p = pk_add(p, pk2(a2, b2));
     x += x2;
     y += y2;
   }
+  a = pk_first(p);
+  b = pk_second(p);
 }
 
 // C^-1 is symmetric and stored as its lower triangle, row by row: entry (i, j), j <= i, at
@@ -293,38 +397,48 @@ __device__ __forceinline__ void untri(int e, int& i, int& j) {
   j = e - tri(i);
 }
 
-// sum_a C^-1[q][idx[a]] b[a] over a < m (skipping idx[a] == skip); BIG (C^-1 in global memory):
-// four independent partial sums so that the gathers of consecutive terms overlap
-template <typename C, bool BIG>
-__device__ __forceinline__ C dot_row(const C* __restrict__ Cp, int q, const int* __restrict__ idx,
-                                     const C* __restrict__ b, int m, int skip) {
-  C s0 = czero<C>();
-  int a = 0;
-  if constexpr (BIG) {
-    constexpr int G = 4;
-    C sp[G];
-#pragma unroll
-    for (int u = 0; u < G; ++u) sp[u] = czero<C>();
-#pragma unroll 1
-    for (; a + G - 1 < m; a += G) {
-      int ix[G];
-      C r[G];
-#pragma unroll
-      for (int u = 0; u < G; ++u) {
-        ix[u] = idx[a + u];
-        r[u] = Cp[pk(q, ix[u])];
+// A lane's walk over the packed triangle, entries e = first, first + L, ...: (i, j) from the
+// block's table below kTriTab entries (the rows of a chain of up to 32 PEs, nearly all of the
+// accepts of the uneven windows), one row carry per step beyond it (rows there have more than L
+// entries). The table replaces a square root and its corrections, about 25 instructions of the
+// 90 that an entry of the accept's pass took.
+constexpr int kTriRows = 32;
+constexpr int kTriTab = kTriRows * (kTriRows + 1) / 2;
+template <int L> struct TriWalk {
+  int i = 0, j = 0;
+  __device__ __forceinline__ void at(const unsigned short* __restrict__ tij, int e) {
+    if (e < kTriTab) {
+      const int t = tij[e];
+      i = t >> 8;
+      j = t & 255;
+    } else {
+      j += L;
+      if (j > i) {
+        j -= i + 1;
+        ++i;
       }
-#pragma unroll
-      for (int u = 0; u < G; ++u)
-        if (ix[u] != skip) sp[u] = cfma(r[u], b[a + u], sp[u]);
     }
-#pragma unroll
-    for (int u = 1; u < G; ++u) sp[0] = cadd(sp[0], sp[u]);
-    s0 = sp[0];
   }
+};
+
+// sum_a C^-1[q][idx[a]] b[a] over a < m, C^-1 in global memory: four independent partial sums so
+// that the gathers of consecutive terms overlap
+template <typename C>
+__device__ __forceinline__ C dot_row4(const C* __restrict__ Cp, int q, const int* __restrict__ idx,
+                                      const C* __restrict__ b, int m) {
+  Pk<C> s01 = pk2(czero<C>(), czero<C>()), s23 = s01;
+  int a = 0;
 #pragma unroll 1
-  for (; a < m; ++a)
-    if (idx[a] != skip) s0 = cfma(Cp[pk(q, idx[a])], b[a], s0);
+  for (; a + 3 < m; a += 4) {
+    C r[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) r[u] = Cp[pk(q, idx[a + u])];
+    s01 = pk_fma(pk2(r[0], r[1]), pk2(b[a], b[a + 1]), s01);
+    s23 = pk_fma(pk2(r[2], r[3]), pk2(b[a + 2], b[a + 3]), s23);
+  }
+  C s0 = cadd(cadd(cadd(pk_first(s01), pk_second(s01)), pk_first(s23)), pk_second(s23));
+#pragma unroll 1
+  for (; a < m; ++a) s0 = cfma(Cp[pk(q, idx[a])], b[a], s0);
   return s0;
 }
 
@@ -390,10 +504,9 @@ __device__ __forceinline__ Sup pe_sup(const DevModel& M, int n, int j) {
 // a_x^T a_q over the window, for x with support s and q = x - o (|o| < Lt), from the prefix table.
 template <typename C, typename TT>
 __device__ __forceinline__ C xcorr(const DevModel& M, const TT* __restrict__ tc, const Sup& s, int o) {
-  const int O = 2 * M.Lt - 1;
-  const TT* base = tc + (size_t)s.ph * M.tcM * O + (o + M.Lt - 1);
-  C v = cload<C>(base[(size_t)s.ihi * O]);
-  if (s.ilo > 0) v = csub(v, cload<C>(base[(size_t)s.ilo * O]));
+  const unsigned O = 2 * M.Lt - 1, row = s.ph * M.tcM;  // at most 64 x 129 x 16383 entries
+  C v = cload<C>(tc[(row + s.ihi) * O + (o + M.Lt - 1)]);
+  if (s.ilo > 0) v = csub(v, cload<C>(tc[(row + s.ilo) * O + (o + M.Lt - 1)]));
   return v;
 }
 
@@ -404,6 +517,7 @@ template <typename T, int L>
 __device__ int pe_birth_search(const DevModel& M, int T_lo, int T_hi, int k0, T base, T target, const Lanes<L> ln) {
   int lo = T_lo, hi = T_hi - 1;
   if ((pe_cphi<T>(M, hi - k0) - base) > target) {
+#pragma unroll 1
     while (lo < hi) {
       const int len = hi - lo + 1;
       const int step = (len + L - 1) / L;
@@ -418,6 +532,7 @@ __device__ int pe_birth_search(const DevModel& M, int T_lo, int T_hi, int k0, T 
     return lo;
   }
   int last = -1;
+#pragma unroll 1
   for (int top = T_hi - 1; top >= T_lo; top -= L) {
     const int j = top - ln.sl;
     const bool ok = j >= T_lo && pe_logphi<T>(M, j - k0) > (T)-INFINITY;
@@ -427,10 +542,68 @@ __device__ int pe_birth_search(const DevModel& M, int T_lo, int T_hi, int k0, T 
   return last;
 }
 
-template <typename T> struct PeRand {
+// cphi(d) without branches (the same values as pe_cphi)
+template <typename T> __device__ __forceinline__ T pe_cphi_clamped(const DevModel& M, int d) {
+  const T v = __ldg(PeTab<T>::cphi(M) + min(max(d + M.D, 0), 2 * M.D));
+  return d < -M.D ? (T)0 : v;
+}
+// The last j of T with phi > 0 for the subgroups with want set, -1 if there is none (a birth search
+// that rounding left without an answer: it runs next to never, so out of line).
+template <typename T, int L>
+__device__ __noinline__ int pe_birth_last(const DevModel& M, int T_lo, int T_hi, int k0, bool want, const Lanes<L> ln) {
+  constexpr int w = L / kSub;
+  const int gi = ln.sl / w, m = ln.sl % w;
+  int last = -1;
+#pragma unroll 1
+  for (int top = T_hi - 1; gballot(want && last < 0 && top >= T_lo, ln); top -= w) {
+    const int j = top - m;
+    const bool ok = want && last < 0 && j >= T_lo && pe_logphi<T>(M, j - k0) > (T)-INFINITY;
+    const unsigned b = (gballot(ok, ln) >> (gi * w)) & ((1u << w) - 1u);
+    if (b) last = top - (__ffs(b) - 1);
+  }
+  return last;
+}
+// The birth search for every subgroup of w lanes at once (subgroups with want = false idle): each
+// lane tests kSub points per round, so that their table loads overlap. u4 is the uniform of the
+// proposal: the target is u4 tot, tot = cphi(T_hi - 1 - k0) - base the mass of T. All lanes of the
+// chain call.
+template <typename T, int L>
+__device__ __forceinline__ int pe_birth_search_sub(const DevModel& M, int T_lo, int T_hi, int k0, T u4, bool want,
+                                                   const Lanes<L> ln) {
+  constexpr int w = L / kSub, P = w * kSub;
+  const int gi = ln.sl / w, m = ln.sl % w;
+  const unsigned sm = ((1u << w) - 1u) << (gi * w);
+  int lo = T_lo, hi = T_hi - 1;
+  const T base = pe_cphi_clamped<T>(M, T_lo - 1 - k0), tot = pe_cphi_clamped<T>(M, hi - k0) - base, target = u4 * tot;
+  const bool found = tot > target;
+#pragma unroll 1
+  while (gballot(want && found && lo < hi, ln)) {
+    const int step = (hi - lo + P) / P;
+    int nf = 0;  // points that are not beyond the target: the first ones
+    T c[kSub];
+#pragma unroll
+    for (int u = 0; u < kSub; ++u)
+      c[u] = pe_cphi_clamped<T>(M, min(hi, lo + (m * kSub + u + 1) * step - 1) - k0);
+#pragma unroll
+    for (int u = 0; u < kSub; ++u) nf += __popc(gballot(!(c[u] - base > target), ln) & sm);
+    lo += nf * step;
+    hi = min(hi, lo + step - 1);
+  }
+  if (gballot(want && !found, ln)) {
+    const int last = pe_birth_last<T, L>(M, T_lo, T_hi, k0, want && !found, ln);
+    if (!found) lo = last;
+  }
+  return lo;
+}
+
+template <typename T, bool MIX> struct PeRand {
   T z1, lu0, u3, u4, z2, lu;  // t0 shift normal, log u2, jump type, PE choice, shift normal, log u7
-  int ep;                     // charge component of a born or updated PE
 };
+template <typename T> struct PeRand<T, true> {
+  T z1, lu0, u3, u4, z2, lu;
+  int ep;  // charge component of a born or updated PE
+};
+template <typename T, bool MIX> __host__ __device__ constexpr size_t pe_rand_bytes() { return sizeof(PeRand<T, MIX>); }
 
 // FP32 value of the uniform ((x >> 11) + 0.5) 2^-53: the odd 54-bit integer 2 (x >> 11) + 1
 // rounded to FP32, times 2^-54 (exact), i.e. the FP64 uniform rounded to FP32 without FP64 work.
@@ -440,60 +613,113 @@ __device__ __forceinline__ float u01_float(uint64_t x) {
 
 // Per-chain statistics (shared memory, written by the group's first lane).
 struct PeStats {
-  long long sN, sN2, sK, sK2;
+  // of the state: the charge summary and the Wasserstein scalars of the PE times and components
+  // (they hold from step q_from on: they change only with z); the sums over the samples of each
+  // and of its square, then log|Sigma| and log L
+  double cur[3], sum[8];
+  static constexpr int kLogdet = 6, kLogL = 7;
   long long St, Se;  // sum of |t_k| (grid units) and of e_k over the PEs of the state
-  double sQ, sQ2, q_cur, logdet, logL, drift_max, wsq;
-  // the Wasserstein scalars of the state (held like q_cur) and their sums
-  double wt_cur, we_cur, sWt, sWt2, sWe, sWe2;
-  unsigned long long alg_words;
-  int acc[3], prop[3], acc_t0, prop_t0, n_refresh, status, q_from, n_acc_refresh, refresh_fail, pad;
+  double drift_max, wsq;
+  int n_refresh, status, q_from, n_acc_refresh, refresh_fail, pad;
 };
+
+// Speculative batches. A chain's step depends on the step before it only where that step was
+// accepted, and most steps are not (accepted: 4 % at one PE, 13 % over the uneven windows, 33 % at
+// 30 PEs). So a chain of up to kSpecPes PEs scores kSpec consecutive steps at once, step i on the
+// i-th of kSpec subgroups of its lanes, all from the same state (each with its own t0: those moves
+// come first, one after the other); the steps up to and including the first accepted one count, the
+// ones behind it are scored again from the new state. Everything a step does with the same values on
+// every lane (the 2x2 algebra, the proposal, the bookkeeping) then runs once per batch instead of
+// once per step: 1077 instead of 1630 warp instructions a step at 8 PEs, and half the code fetched.
+// The decisions and every rounding are those of the one-by-one steps: a subgroup adds up the L
+// lanes' partial sums in the same order (each of its lanes holds kSpec of them). Four steps: with
+// eight the batch's loops are twice as long, and wait for instructions too (low occupancy 106 ms
+// against 104, one event 5.97 against 5.22). Up to 32 PEs: beyond, the entries scored for steps
+// that do not count cost what the batch saves. 20 000 uneven windows x 2000 steps: 120 -> 110 ms,
+// 100 000 low-occupancy chains x 1000: 134 -> 103 ms, 256 FP64 chains x 1000: 13.7 -> 9.8 ms.
+constexpr int kSpec = kSub;
+constexpr int kSpecPes = 32;   // most PEs of a chain scored this way (indices in W.ix())
+constexpr int kCounts = 8;     // integer counts of a chain, per subgroup (PeChain::cnt)
+
+// A step's addition to count q: sums over the samples after burn-in of N, N^2, k0 and k0^2, the
+// algorithmic words, then pairs of counters: proposed births | deaths, accepted births | deaths,
+// accepted updates | accepted t0 moves (a chain's other proposals follow from its step count).
+__device__ __forceinline__ unsigned long long count_of(int q, int N, int k0, bool past, unsigned words, int jump,
+                                                       bool applied, bool t0_acc) {
+  const int a = (q & 2) ? k0 : N, b = (q & 1) ? a : 1;
+  const unsigned long long jp = jump == 0 ? 1ull : (jump == 1 ? 1ull << 32 : 0ull);
+  const unsigned long long tail = q == 4 ? (unsigned long long)words
+                                  : q == 5 ? jp
+                                  : q == 6 ? (applied ? jp : 0ull)
+                                           : (applied && jump == 2 ? 1ull : 0ull) + (t0_acc ? 1ull << 32 : 0ull);
+  return q < 4 ? (past ? (unsigned long long)((long long)a * (long long)b) : 0ull) : tail;
+}
 
 __host__ __device__ inline size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-// Per-chain shared memory. C is the state type (16 bytes in FP64 mode, 8 in FP32 mode).
-template <typename T> struct PeChain {
-  using C = typename PeTab<T>::C;
-  PeStats* st;
-  PeRand<T>* rnd;  // draws of the next L steps [L]
-  int* list;   // PE grid indices [n_cap]
-  unsigned char* le;  // PE charge components [n_cap]
-  int* ovi;    // PEs overlapping the proposed one [n_cap]
-  C* ovb;      // their inner products with it [n_cap]
-  C* v;        // C^-1 A^T y [n_cap]
-  C* cv;       // row k of C^-1 / C^-1 b [n_cap]
-  C* uv;       // second work vector [n_cap]
-  T* y;        // residual [n_alloc]
-  T* lPhi;     // log(Phi_T(t0) g) on the chain's t0 grid [win_extra]
-  C* Cs;       // C^-1 tile: packed triangle of Ns PEs
-};
-template <typename T, int L> __host__ __device__ inline size_t pe_chain_bytes(int n_cap, int n_alloc, int win_extra, int Ns) {
-  constexpr size_t cs = sizeof(typename PeTab<T>::C);
-  return a16(sizeof(PeStats)) + a16(sizeof(PeRand<T>) * L) + 2 * a16(sizeof(int) * n_cap) + a16((size_t)n_cap) +
-         4 * a16(cs * (size_t)n_cap) + a16(sizeof(T) * n_alloc) + a16(sizeof(T) * win_extra) +
-         a16(cs * (size_t)tri(Ns));
-}
-// Block tables: the SER, log(i) and 1 / i (i <= n_cap + 1).
+// The CTA's dynamic shared memory: the block tables, then a block per chain. Everything in it is
+// addressed by 32-bit offsets from this symbol, so that the compiler sees shared memory also in
+// the out-of-line functions (generic 64-bit pointers there cost two registers each and about a
+// third more code, which is what binds chains with few PEs: the step has to stay in the SM's
+// 32 KB instruction cache).
+extern __shared__ __align__(16) unsigned char pe_smem[];
+
+// Block tables: (i, j) of the first packed entries, the SER, log(i) and 1 / i (i <= n_cap + 1).
+constexpr unsigned kTabBytes = (sizeof(unsigned short) * kTriTab + 15) & ~15u;
 template <typename T> __host__ __device__ inline size_t pe_block_bytes(const DevModel& M) {
-  return a16(sizeof(T) * M.Lt) + a16(sizeof(T) * (M.n_cap + 2)) + a16(sizeof(double) * (M.n_cap + 2));
+  return kTabBytes + a16(sizeof(T) * M.Lt) + a16(sizeof(T) * (M.n_cap + 2)) + a16(sizeof(double) * (M.n_cap + 2));
 }
-template <typename T, int L> __device__ PeChain<T> pe_carve(unsigned char* p, int n_cap, int n_alloc, int win_extra, int Ns) {
+__device__ __forceinline__ unsigned short* pe_tij() { return reinterpret_cast<unsigned short*>(pe_smem); }
+template <typename T> __device__ __forceinline__ T* pe_V() { return reinterpret_cast<T*>(pe_smem + kTabBytes); }
+
+// Per-chain shared memory. C is the state type (16 bytes in FP64 mode, 8 in FP32 mode).
+template <typename T, bool BIG, int L, bool MIX> struct PeChain {
   using C = typename PeTab<T>::C;
-  PeChain<T> W;
-  size_t o = 0;
-  W.st = reinterpret_cast<PeStats*>(p + o); o += a16(sizeof(PeStats));
-  W.rnd = reinterpret_cast<PeRand<T>*>(p + o); o += a16(sizeof(PeRand<T>) * L);
-  W.list = reinterpret_cast<int*>(p + o); o += a16(sizeof(int) * n_cap);
-  W.le = p + o; o += a16((size_t)n_cap);
-  W.ovi = reinterpret_cast<int*>(p + o); o += a16(sizeof(int) * n_cap);
-  W.ovb = reinterpret_cast<C*>(p + o); o += a16(sizeof(C) * (size_t)n_cap);
-  W.v = reinterpret_cast<C*>(p + o); o += a16(sizeof(C) * (size_t)n_cap);
-  W.cv = reinterpret_cast<C*>(p + o); o += a16(sizeof(C) * (size_t)n_cap);
-  W.uv = reinterpret_cast<C*>(p + o); o += a16(sizeof(C) * (size_t)n_cap);
-  W.y = reinterpret_cast<T*>(p + o); o += a16(sizeof(T) * n_alloc);
-  W.lPhi = reinterpret_cast<T*>(p + o); o += a16(sizeof(T) * win_extra);
-  W.Cs = reinterpret_cast<C*>(p + o);
-  return W;
+  unsigned o;    // the chain's block
+  unsigned vb;   // bytes of a vector of n_cap state values
+  unsigned lb;   // bytes of the PE list
+  unsigned yb;   // bytes of the residual
+  unsigned pb;   // bytes of log Phi
+  static constexpr unsigned kCnt = (sizeof(PeStats) + 15) & ~15u, kIx = kCnt + 8 * kSpec * kCounts,
+                            kRnd = kIx + (BIG ? 0 : kSpec * kSpecPes),
+                            kVec = (kRnd + (unsigned)sizeof(PeRand<T, MIX>) * L + 15) & ~15u;
+  template <typename E> __device__ __forceinline__ E* at(unsigned b) const {
+    return reinterpret_cast<E*>(pe_smem + (o + b));
+  }
+  __device__ __forceinline__ PeStats& st() const { return *at<PeStats>(0); }
+  // counts [kSpec][kCounts]
+  __device__ __forceinline__ unsigned long long* cnt() const { return at<unsigned long long>(kCnt); }
+  // batch: PEs overlapping each subgroup's proposed one [kSpec][kSpecPes]
+  __device__ __forceinline__ unsigned char* ix() const { return at<unsigned char>(kIx); }
+  // draws of the next L steps
+  __device__ __forceinline__ PeRand<T, MIX>* rnd() const { return at<PeRand<T, MIX>>(kRnd); }
+  __device__ __forceinline__ C* v() const { return at<C>(kVec); }  // C^-1 A^T y
+  // four work vectors (BIG: three and a list of indices). In a batch, subgroup i keeps the
+  // proposed PE's inner products b in the i-th. Otherwise: b over the overlapping PEs (the accept
+  // then keeps u' / delta there), row k of C^-1, C^-1 b, and b's indices (then c / -gamma)
+  __device__ __forceinline__ C* work(int i) const { return at<C>(kVec + (1 + i) * vb); }
+  __device__ __forceinline__ C* ovb() const { return work(0); }
+  __device__ __forceinline__ C* cv() const { return work(1); }
+  __device__ __forceinline__ C* uv() const { return work(2); }
+  __device__ __forceinline__ int* ovi() const { return at<int>(kVec + 4 * vb); }
+  __device__ __forceinline__ C* cvn() const { return work(3); }  // not BIG
+  __device__ __forceinline__ int* list() const { return at<int>(tail()); }  // PE grid indices [n_cap]
+  __device__ __forceinline__ unsigned tail() const { return kVec + 4 * vb + (BIG ? lb : vb); }
+  // residual [n_alloc], then log(Phi_T(t0) g) on the chain's t0 grid [win_extra], the C^-1 tile
+  // (packed triangle of Ns PEs) and the PEs' charge components [n_cap] (mixture only)
+  __device__ __forceinline__ T* y() const { return at<T>(tail() + lb); }
+  __device__ __forceinline__ T* lPhi() const { return at<T>(tail() + lb + yb); }
+  __device__ __forceinline__ unsigned char* le() const { return at<unsigned char>(tail() + lb + yb + pb); }
+  __device__ __forceinline__ C* Cs(int n_cap) const {
+    return at<C>(tail() + lb + yb + pb + (MIX ? (unsigned)a16((size_t)n_cap) : 0u));
+  }
+};
+template <typename T, bool BIG, int L, bool MIX>
+__host__ __device__ inline size_t pe_chain_bytes(int n_cap, int n_alloc, int win_extra, int Ns) {
+  constexpr size_t cs = sizeof(typename PeTab<T>::C);
+  return PeChain<T, BIG, L, MIX>::kVec + 4 * a16(cs * (size_t)n_cap) + a16((BIG ? sizeof(int) : cs) * (size_t)n_cap) +
+         a16(sizeof(int) * n_cap) + a16(sizeof(T) * n_alloc) + a16(sizeof(T) * win_extra) +
+         (MIX ? a16((size_t)n_cap) : 0) + a16(cs * (size_t)tri(Ns));
 }
 
 // Global per-chain slots (one per resident chain of the launch).
@@ -517,29 +743,31 @@ __host__ __device__ inline size_t pe_ws_doubles(int n_cap) {
   return pe_ws_a2((size_t)n_cap * n_cap) + (2 + 2 * kSweepBlock) * pe_ws_a2(n_cap) + kSweepBlock * kSweepBlock;
 }
 
-// Hold of the state's summaries: the charge summary q_cur and the Wasserstein scalars wt_cur,
-// we_cur hold from step q_from on (they change only with z); close the hold at step s.
-__device__ __forceinline__ void close_hold(PeStats& S, int s, int burn_in) {
-  const int from = max(S.q_from, burn_in);
-  if (s > from) {
-    const double c = (double)(s - from);
-    S.sQ += S.q_cur * c;
-    S.sQ2 += S.q_cur * S.q_cur * c;
-    S.sWt += S.wt_cur * c;
-    S.sWt2 += S.wt_cur * S.wt_cur * c;
-    S.sWe += S.we_cur * c;
-    S.sWe2 += S.we_cur * S.we_cur * c;
+// Close the hold of the state's summaries at step s and, where a move was accepted (dT, dnu: its
+// changes of log|Sigma| and log L), add these: a lane per sum, so that the FP64 operations (64
+// issue cycles each on this part, however few lanes take part) are done once for all of them.
+template <typename T>
+__device__ __forceinline__ void close_hold(PeStats& S, int s, int burn_in, bool accepted, T dT, T dnu, int sl) {
+  if (sl < 8) {
+    const int held = s - max(S.q_from, burn_in);
+    double x = sl < 6 ? S.cur[sl >> 1] : (double)(sl == 6 ? dT : dnu);
+    if (sl < 6 && (sl & 1)) x = x * x;
+    if (sl < 6 ? held > 0 : accepted) S.sum[sl] = fma(x, sl < 6 ? (double)held : 1.0, S.sum[sl]);
   }
 }
-
-// The Wasserstein scalars of a state with N PEs (the convergence check of Sec. 3.2): with a
-// dummy PE at t = 0, e = 0 added, the 1-Wasserstein distance from the sequence to the dummy
-// alone is the mean of |t| (or of e) over the N + 1 points.
-// inv1[i] = 1 / i (a block table, so that no FP64 division runs in the step loop).
-__device__ __forceinline__ void set_wasserstein(PeStats& S, double g, int N, const double* inv1) {
-  const double inv = inv1[N + 1];
-  S.wt_cur = g * (double)S.St * inv;
-  S.we_cur = (double)S.Se * inv;
+// The summaries of a state with N PEs, a lane per value: the charge sum_k (mu_k + v_k), given
+// qs = sum v_k and ms = mu (dynode: times N) or sum_k mu_k (mixture), and the Wasserstein scalars
+// (the convergence check of Sec. 3.2): with a dummy PE at t = 0, e = 0 added, the 1-Wasserstein
+// distance from the sequence to the dummy alone is the mean of |t| (or of e) over the N + 1
+// points. inv1[i] = 1 / i (a block table, so that no FP64 division runs in the step loop).
+template <bool MIX>
+__device__ __forceinline__ void set_summaries(PeStats& S, double g, int N, double ms, double qs, const double* inv1,
+                                              int sl) {
+  if (sl < 3) {
+    const long long n = sl == 0 ? (MIX ? 1 : N) : (sl == 1 ? S.St : S.Se);
+    const double x = fma((double)n, sl == 0 ? ms : (sl == 1 ? g : 1.0), sl == 0 ? qs : 0.0);
+    S.cur[sl] = sl == 0 ? x : x * inv1[N + 1];
+  }
 }
 
 // lambda_FSMP at the chain end, out of line: the estimator's code stays out of the step loop's
@@ -558,7 +786,7 @@ struct RefreshOut {
 // ok = 0 (state untouched) if C is not numerically positive definite. Arguments are passed by
 // value (no address of the caller's locals escapes, so they stay in registers).
 template <typename T, bool BIG, int L, bool MIX>
-__device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T> W, typename PeTab<T>::C* Cp,
+__device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T, BIG, L, MIX> W, typename PeTab<T>::C* Cp,
                                               double* ws, int n_cap, const float* w, double wsq, int n,
                                               int N, const Lanes<L> ln) {
   using C = typename PeTab<T>::C;
@@ -583,21 +811,21 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
   constexpr int RC = BIG ? 4 : 1, RG = BIG ? 4 : 1;
 #pragma unroll 1
   for (int j = ln.sl; j < N; j += L) {
-    const int jj = W.list[j];
+    const int jj = W.list()[j];
 #pragma unroll 1
     for (int i0 = j; i0 < N; i0 += RC) {
       double c[RC];
 #pragma unroll
       for (int q = 0; q < RC; ++q) {
         const int i = min(i0 + q, N - 1);
-        const int ji = W.list[i];
+        const int ji = W.list()[i];
         const int o = ji - jj;
         c[q] = (o > -M.Lt && o < M.Lt) ? xcorr<double>(M, M.tc64, pe_sup(M, n, ji), o) : 0.0;
       }
 #pragma unroll
       for (int q = 0; q < RC; ++q) {
         const int i = i0 + q;
-        if (i < N) A[(size_t)i * ws_ld + j] = c[q] + (j == i ? (mix ? M.cm_r[W.le[i]] : r) : 0.0);
+        if (i < N) A[(size_t)i * ws_ld + j] = c[q] + (j == i ? (mix ? M.cm_r[W.le()[i]] : r) : 0.0);
       }
     }
   }
@@ -608,7 +836,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
   double awt = 0.0, rst = 0.0;
 #pragma unroll 1
   for (int k = ln.sl; k < N; k += L) {
-    const Sup s = pe_sup(M, n, W.list[k]);
+    const Sup s = pe_sup(M, n, W.list()[k]);
     // the loops' loads go four at a time ahead of their (unchanged) sums
     double a0 = 0.0, a1 = 0.0;
     int i = s.ilo;
@@ -635,7 +863,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
     auto c_kj = [&](int j) { return *(j <= k ? A + (size_t)k * ws_ld + j : A + (size_t)j * ws_ld + k); };
     int j = 0;
     if (mix) {
-      const int ek = W.le[k];
+      const int ek = W.le()[k];
       const double mk = M.cm_mu[ek];
       double hs = -M.cm_r[ek] * mk;  // (A^T A m)_k = sum_j C_kj m_j - r_k m_k
 #pragma unroll 1
@@ -644,13 +872,13 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           cc[u] = c_kj(j + u);
-          mm[u] = M.cm_mu[W.le[j + u]];
+          mm[u] = M.cm_mu[W.le()[j + u]];
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) hs = fma(cc[u], mm[u], hs);
       }
 #pragma unroll 1
-      for (; j < N; ++j) hs = fma(c_kj(j), M.cm_mu[W.le[j]], hs);
+      for (; j < N; ++j) hs = fma(c_kj(j), M.cm_mu[W.le()[j]], hs);
       h[k] = aw - hs;
       awt = fma(mk, aw, awt);
       rst = fma(mk, hs, rst);
@@ -684,24 +912,24 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
     __syncwarp(ln.gm);
 #pragma unroll 1
     for (int k = 0; k < N; ++k) {
-      const Sup s = pe_sup(M, n, W.list[k]);
-      const double mk = mix ? -M.cm_mu[W.le[k]] : -mu;
+      const Sup s = pe_sup(M, n, W.list()[k]);
+      const double mk = mix ? -M.cm_mu[W.le()[k]] : -mu;
 #pragma unroll 1
       for (int i = s.ilo + ln.sl; i < s.ihi; i += L) yd[s.w0 + i] = fma(mk, V[s.ph + i * M.R], yd[s.w0 + i]);
       __syncwarp(ln.gm);
     }
 #pragma unroll 1
-    for (int x = ln.sl; x < n; x += L) W.y[x] = (T)yd[x];
+    for (int x = ln.sl; x < n; x += L) W.y()[x] = (T)yd[x];
   } else {
 #pragma unroll 1
     for (int x = ln.sl; x < n; x += L) {
       double yv = (double)w[x];
 #pragma unroll 1
       for (int k = 0; k < N; ++k) {
-        const int idx = x * M.R - W.list[k];
-        if (idx >= 0 && idx < M.Lt) yv = fma(mix ? -M.cm_mu[W.le[k]] : -mu, V[idx], yv);
+        const int idx = x * M.R - W.list()[k];
+        if (idx >= 0 && idx < M.Lt) yv = fma(mix ? -M.cm_mu[W.le()[k]] : -mu, V[idx], yv);
       }
-      W.y[x] = (T)yv;
+      W.y()[x] = (T)yv;
     }
   }
   __syncwarp(ln.gm);
@@ -887,9 +1115,9 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
   double vd = 0.0, va = 0.0;
 #pragma unroll 1
   for (int i = ln.sl; i < N; i += L) {
-    vd = fmax(vd, fabs(rowk[i] - c64(W.v[i])));
+    vd = fmax(vd, fabs(rowk[i] - c64(W.v()[i])));
     va = fmax(va, fabs(rowk[i]));
-    W.v[i] = cfrom64<C>(rowk[i]);
+    W.v()[i] = cfrom64<C>(rowk[i]);
   }
   dmax = wmax(dmax, ln); amax = wmax(amax, ln); vd = wmax(vd, ln); va = wmax(va, ln);
   __syncwarp(ln.gm);
@@ -898,7 +1126,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
   if (mix) {
     lrs = 0.0;
 #pragma unroll 1
-    for (int k = ln.sl; k < N; k += L) lrs += M.cm_lr[W.le[k]];
+    for (int k = ln.sl; k < N; k += L) lrs += M.cm_lr[W.le()[k]];
     lrs = wsum(lrs, ln);
   }
   out.ok = 1;
@@ -912,7 +1140,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
 template <typename C> struct PeMove {
   int jump, kk, jp, jm, np;
   int em, ep;  // charge components of the removed and the new PE
-  C aa, quad, bv, vk, ay;
+  C aa, vk, ay;
   Sup sp;
 };
 
@@ -923,22 +1151,23 @@ template <typename C> struct AcceptOut {
   C idl;  // 1 / delta, delta the Schur complement of the new PE (birth, update)
 };
 
-// Apply an accepted move to C^-1, v, y and the PE list (out of line: it runs on a minority of
-// steps and keeps the per-step code compact). Returns the new N, and the new C^-1 storage when
-// it moves from the shared tile (capacity cap PEs) to the global slot (n_cap PEs).
+// Apply an accepted move to C^-1, v, y and the PE list. Returns the new N, and the new C^-1 storage
+// when it moves from the shared tile (capacity cap PEs) to the global slot (n_cap PEs). Inlined in
+// the step loop (the call's moves and the model constants' generic loads cost it 4 %).
 template <typename T, bool BIG, int L, bool MIX>
-__device__ __noinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevModel& M, const PeChain<T> W, const T* Vs,
+__device__ __forceinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevModel& M, const PeChain<T, BIG, L, MIX> W,
                                                                   typename PeTab<T>::C* Cp, int cap,
                                                                   typename PeTab<T>::C* Cg,
                                                                   const PeMove<typename PeTab<T>::C> mv, int n, int N,
                                                                   const Lanes<L> ln) {
-  // One form for the three moves. With c = row k of C^-1 (death, update), gamma = c_k, and
-  // u' = C_-^-1 b~ (birth, update: C_- is C without PE k for an update, C itself for a birth;
-  // b~ is b without its k entry), delta = r + |a_+|^2 - b~^T u':
+  // With c = row k of C^-1 (death, update), gamma = c_k, and u' = C_-^-1 b~ (birth, update: C_- is
+  // C without PE k for an update, C itself for a birth; b~ is b without its k entry),
+  // delta = r + |a_+|^2 - b~^T u':
   //   C'_ij = C_{m(i) m(j)} - c_m(i) c_m(j) / gamma + u'_i u'_j / delta   (i, j != s),
   //   C'_is = -u'_i / delta,  C'_ss = 1 / delta,
   // where s is the slot of the new PE (N for a birth, k for an update; none for a death) and
-  // m moves the last PE into slot k for a death (identity otherwise). v changes the same way.
+  // m moves the last PE into slot k for a death (identity otherwise). A birth has no c term, a
+  // death no u' term. v changes the same way.
   // The removed PE has mean mu_- (component em), the new one mean mu_+ and r_+ (component ep).
   using C = typename PeTab<T>::C;
   const int em = MIX ? mv.em : 0, ep = MIX ? mv.ep : 0;
@@ -946,74 +1175,94 @@ __device__ __noinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevModel
   const T mumT = CmT<T>::mu(M, em), mupT = CmT<T>::mu(M, ep);
   const int R = M.R, np = mv.np, kk = mv.kk, jump = mv.jump;
   const bool has_m = jump != 0, has_p = jump != 1;
-  const int skip = jump == 2 ? kk : -1;
   const int Nout = N + (jump == 0 ? 1 : (jump == 1 ? -1 : 0));
   const int s = jump == 0 ? N : (jump == 2 ? kk : -1);
   const int last = N - 1;
-  // vectors: c (cv; zero for a birth) and C^-1 b~ (uv; zero for a death). The passes below
-  // always apply both terms, so that they have no branches on the move type.
-  const int krow = has_m ? kk : 0;
-  const int npu = has_p ? np : 0;
-  if constexpr (BIG) {
-#pragma unroll 1
-    for (int i = ln.sl; i < N; i += L) {
-      const C ci = Cp[pk(krow, i)];
-      W.cv[i] = has_m ? ci : czero<C>();
-      W.uv[i] = dot_row<C, BIG>(Cp, i, W.ovi, W.ovb, npu, skip);
-    }
-  } else {
-    // s lanes per row (s N <= L), each summing every s-th term of the row's product with b~,
-    // then a butterfly over the s lanes: the dependent chain of a row is npu / s terms long
-    int s = 1;
-    while (s < 8 && 2 * s * N <= L) s <<= 1;
-    const int rq = ln.sl / s, qq = ln.sl - rq * s, rpp = L / s;
-#pragma unroll 1
-    for (int i0 = 0; i0 < N; i0 += rpp) {
-      const int i = i0 + rq;
-      C acc = czero<C>();
-      if (i < N) {
-#pragma unroll 1
-        for (int a = qq; a < npu; a += s)
-          if (W.ovi[a] != skip) acc = cfma(Cp[pk(i, W.ovi[a])], W.ovb[a], acc);
-      }
-#pragma unroll 1
-      for (int o = 1; o < s; o <<= 1) acc = cadd(acc, cshfl_xor<L>(acc, o, ln.gm));
-      if (i < N && qq == 0) {
-        W.cv[i] = has_m ? Cp[pk(krow, i)] : czero<C>();
-        W.uv[i] = acc;
-      }
-    }
-  }
-  if (ln.sl == 0 && jump == 0) { W.cv[N] = czero<C>(); W.uv[N] = czero<C>(); }  // slot N of a birth (N < n_cap)
-  __syncwarp(ln.gm);
-  C ig = czero<C>(), idl = czero<C>(), t = czero<C>(), fv = czero<C>();
-  if (has_m) {
-    ig = crcp(W.cv[kk]);
-    fv = cmul(cadd(mv.vk, mum), ig);
-  }
+  C* const cvn = BIG ? W.cv() : W.cvn();  // c / -gamma (BIG has no room for it: taken per entry)
+  C* const uvd = W.ovb();  // u' / delta, once b is no longer read
+  const T* const Vs = pe_V<T>();
+  const unsigned short* const tij = pe_tij();
+  C ig = czero<C>(), idl = czero<C>(), t = czero<C>(), fv = czero<C>(), nig = czero<C>();
+  C bvf = czero<C>(), bk = czero<C>(), wk = czero<C>();
   if (has_p) {
     // b^T v in full state precision (the scoring used an FP32 sum) and, for an update, the
-    // entry of b for PE k, in one butterfly
-    C bvf = czero<C>(), bk = czero<C>();
+    // entry of b for PE k, in one butterfly; then b~ in b's place
 #pragma unroll 1
     for (int a = ln.sl; a < np; a += L) {
-      bvf = cfma(W.ovb[a], W.v[W.ovi[a]], bvf);
-      if (jump == 2 && W.ovi[a] == kk) bk = W.ovb[a];
+      bvf = cfma(W.ovb()[a], W.v()[W.ovi()[a]], bvf);
+      if (opaque(jump == 2) && W.ovi()[a] == kk) {
+        bk = W.ovb()[a];
+        W.ovb()[a] = czero<C>();
+      }
     }
-    const C wk = jump == 2 ? W.uv[kk] : czero<C>();  // read by every lane before the butterfly
-    csum2(bvf, bk, ln);
+    csum2_m(bvf, bk, np, ln);
+    if constexpr (BIG) {
+      __syncwarp(ln.gm);
+#pragma unroll 1
+      for (int i = ln.sl; i < N; i += L) W.uv()[i] = dot_row4<C>(Cp, i, W.ovi(), W.ovb(), np);
+    } else if (N > L) {
+      // two rows per lane, i and i + L
+      __syncwarp(ln.gm);
+#pragma unroll 1
+      for (int i = ln.sl; i < N; i += 2 * L) {
+        const int i2 = min(i + L, N - 1);
+        Pk<C> acc = pk2(czero<C>(), czero<C>());
+#pragma unroll 1
+        for (int a = 0; a < np; ++a) {
+          const int q = W.ovi()[a];
+          const C b = W.ovb()[a];
+          acc = pk_fma(pk2(Cp[pk(i, q)], Cp[pk(i2, q)]), pk2(b, b), acc);
+        }
+        W.uv()[i] = pk_first(acc);
+        if (i + L < N) W.uv()[i + L] = pk_second(acc);
+      }
+    } else {
+      // 2^ls lanes per row (2^ls N <= L), each summing every 2^ls-th term of the row's product with
+      // b~, then a butterfly over them: the dependent chain of a row is np / 2^ls terms long
+      int ls = 0;
+#pragma unroll 1
+      while (ls < 3 && (2 * N << ls) <= L) ++ls;
+      const int rq = ln.sl >> ls, qq = ln.sl & ((1 << ls) - 1), rpp = L >> ls;
+      __syncwarp(ln.gm);
+#pragma unroll 1
+      for (int i0 = 0; i0 < N; i0 += rpp) {
+        const int i = i0 + rq;
+        C acc = czero<C>();
+        if (i < N) {
+#pragma unroll 1
+          for (int a = qq; a < np; a += 1 << ls) acc = cfma(Cp[pk(i, W.ovi()[a])], W.ovb()[a], acc);
+        }
+#pragma unroll 1
+        for (int o = 1; o < 1 << ls; o <<= 1) acc = cadd(acc, cshfl_xor<L>(acc, o, ln.gm));
+        if (i < N && qq == 0) W.uv()[i] = acc;
+      }
+    }
+    if (ln.sl == 0 && jump == 0) W.uv()[N] = czero<C>();  // slot N of a birth (N < n_cap)
+  }
+  if (has_m) {
+#pragma unroll 1
+    for (int i = ln.sl; i < N; i += L) W.cv()[i] = Cp[pk(kk, i)];
+    __syncwarp(ln.gm);
+    ig = crcp(W.cv()[kk]);
+    nig = cneg(ig);
+    fv = cmul(cadd(mv.vk, mum), ig);
+  } else {
+    __syncwarp(ln.gm);
+  }
+  if (has_p) {
     if (jump == 2) {
       // u' = w - c w_k / gamma on the system without PE k
+      wk = W.uv()[kk];
       const C wkg = cneg(cmul(wk, ig));
+      __syncwarp(ln.gm);  // every lane has read w_k
 #pragma unroll 1
-      for (int i = ln.sl; i < N; i += L) W.uv[i] = (i == kk) ? czero<C>() : cfma(W.cv[i], wkg, W.uv[i]);
+      for (int i = ln.sl; i < N; i += L) W.uv()[i] = (i == kk) ? czero<C>() : cfma(W.cv()[i], wkg, W.uv()[i]);
       __syncwarp(ln.gm);
     }
     C bu = czero<C>();
 #pragma unroll 1
-    for (int a = ln.sl; a < np; a += L)
-      if (W.ovi[a] != skip) bu = cfma(W.ovb[a], W.uv[W.ovi[a]], bu);
-    bu = csum(bu, ln);
+    for (int a = ln.sl; a < np; a += L) bu = cfma(W.ovb()[a], W.uv()[W.ovi()[a]], bu);
+    bu = csum_m(bu, np, ln);
     idl = crcp(csub(cadd(rrp, mv.aa), bu));
     // t = (b~^T v_- - mu_+ b~^T u' - h_new) / delta with v_- = v after removing PE k and h_new
     // the new PE's a^T y on the final residual (PE k removed, the new PE added)
@@ -1021,108 +1270,178 @@ __device__ __noinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevModel
     const C hnew = csub(cadd(mv.ay, cmul(mum, bk)), cmul(mup, mv.aa));
     t = cmul(csub(csub(bvm, cmul(mup, bu)), hnew), idl);
   }
+  // the factors c / -gamma and u' / delta, once per PE instead of once per entry
+  __syncwarp(ln.gm);  // b and its indices are read
+#pragma unroll 1
+  for (int i = ln.sl; i <= N; i += L) {
+    if (!BIG && opaque(has_m) && i < N) cvn[i] = cmul(W.cv()[i], nig);
+    if (opaque(has_p) && i < Nout) uvd[i] = cmul(W.uv()[i], idl);
+  }
   if (jump == 0 && N + 1 > cap && Cp != Cg) {  // the tile is full: move C^-1 to the global slot
 #pragma unroll 1
     for (int e = ln.sl; e < tri(N); e += L) Cg[e] = Cp[e];
     Cp = Cg;
     cap = M.n_cap;
-    __syncwarp(ln.gm);
   }
+  __syncwarp(ln.gm);
   // C^-1 in place over the packed triangle, all lanes on consecutive entries. A pass reads an
   // entry only where it writes it, or in the last row for a death (which it does not write).
-  const C nig = cneg(ig);
   const int kmap = jump == 1 ? kk : -1;  // the slot the last PE moves into
   const int ne = tri(Nout);               // rows 0 .. Nout-1
-  int e0 = 0;
+  auto src = [&](int i, int j) { return pk(i == kmap ? last : i, j == kmap ? last : j); };
+  auto update2 = [&](int i, int j, C& x, int i2, int j2, C& x2) {
+    Pk<C> y = pk2(x, x2);
+    if (opaque(has_m)) {
+      Pk<C> cj = pk2(cvn[j == kmap ? last : j], cvn[j2 == kmap ? last : j2]);
+      if constexpr (BIG) cj = pk_mul(cj, pk2(nig, nig));
+      y = pk_fma(pk2(W.cv()[i == kmap ? last : i], W.cv()[i2 == kmap ? last : i2]), cj, y);
+    }
+    if (opaque(has_p)) y = pk_fma(pk2(W.uv()[i], W.uv()[i2]), pk2(uvd[j], uvd[j2]), y);
+    x = pk_first(y);
+    x2 = pk_second(y);
+    if (opaque(has_p)) {
+      if (i == s || j == s) x = i == j ? idl : cneg(uvd[i == s ? j : i]);
+      if (i2 == s || j2 == s) x2 = i2 == j2 ? idl : cneg(uvd[i2 == s ? j2 : i2]);
+    }
+  };
+  TriWalk<L> tw;
+  int e = ln.sl;
   if constexpr (BIG) {
     // C^-1 in the global slot: four entries per lane and pass, all read before any is written
     // (each read is the entry itself or one in the unwritten last row), so that the loads of a
     // pass overlap
 #pragma unroll 1
-    for (; e0 + 4 * L <= ne; e0 += 4 * L) {
+    for (; e - ln.sl + 4 * L <= ne; e += 4 * L) {
       int ii[4], jj[4];
-      C old[4];
+      C x[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        untri(e0 + q * L + ln.sl, ii[q], jj[q]);
-        const int mi = (ii[q] == kmap) ? last : ii[q], mj = (jj[q] == kmap) ? last : jj[q];
-        old[q] = Cp[pk(mi, mj)];
+        tw.at(tij, e + q * L);
+        ii[q] = tw.i;
+        jj[q] = tw.j;
+        x[q] = Cp[src(tw.i, tw.j)];
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = ii[q], j = jj[q];
-        const int mi = (i == kmap) ? last : i, mj = (j == kmap) ? last : j;
-        const C val = cfma(W.uv[i], cmul(W.uv[j], idl), cfma(W.cv[mi], cmul(W.cv[mj], nig), old[q]));
-        const C sv = (i == s && j == s) ? idl : cneg(cmul(W.uv[i == s ? j : i], idl));
-        Cp[e0 + q * L + ln.sl] = (i == s || j == s) ? sv : val;
-      }
+      for (int q = 0; q < 4; q += 2) update2(ii[q], jj[q], x[q], ii[q + 1], jj[q + 1], x[q + 1]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) Cp[e + q * L] = x[q];
     }
   }
+  // entries e and e + L of a lane, both read before either is written
 #pragma unroll 1
-  for (int e = e0 + ln.sl; e < ne; e += L) {
-    int i, j;
-    untri(e, i, j);
-    const int mi = (i == kmap) ? last : i, mj = (j == kmap) ? last : j;
-    const C old = Cp[pk(mi, mj)];
-    const C val = cfma(W.uv[i], cmul(W.uv[j], idl), cfma(W.cv[mi], cmul(W.cv[mj], nig), old));
-    const C sv = (i == s && j == s) ? idl : cneg(cmul(W.uv[i == s ? j : i], idl));
-    Cp[e] = (i == s || j == s) ? sv : val;
+  for (; e < ne; e += 2 * L) {
+    tw.at(tij, e);
+    const int i = tw.i, j = tw.j;
+    const bool two = e + L < ne;
+    if (two) tw.at(tij, e + L);
+    C x = Cp[src(i, j)], x2 = Cp[src(tw.i, tw.j)];
+    update2(i, j, x, tw.i, tw.j, x2);
+    Cp[e] = x;
+    if (two) Cp[e + L] = x2;
   }
   // v' = v_m - c_m fv + (t - mu_+) u', v'_s = -t
   const C tm = csub(t, mup), nfv = cneg(fv);
 #pragma unroll 1
   for (int i = ln.sl; i < Nout; i += L) {
     const int mi = (i == kmap) ? last : i;
-    const C val = cfma(tm, W.uv[i], cfma(W.cv[mi], nfv, W.v[mi]));
-    W.v[i] = (i == s) ? cneg(t) : val;
+    C x = i < N ? W.v()[mi] : czero<C>();
+    if (opaque(has_m)) x = cfma(W.cv()[mi], nfv, x);
+    if (opaque(has_p)) x = i == s ? cneg(t) : cfma(tm, W.uv()[i], x);
+    W.v()[i] = x;
   }
   // residual and PE list
   unsigned long long wds = (unsigned long long)N * np + 2ull * tri(Nout) + 2ull * Nout;
   if (has_m) {
     const Sup sm = pe_sup(M, n, mv.jm);
 #pragma unroll 1
-    for (int i = sm.ilo + ln.sl; i < sm.ihi; i += L) W.y[sm.w0 + i] += mumT * Vs[sm.ph + i * R];
+    for (int i = sm.ilo + ln.sl; i < sm.ihi; i += L) W.y()[sm.w0 + i] += mumT * Vs[sm.ph + i * R];
     wds += 2 * (sm.ihi - sm.ilo) + N;
     __syncwarp(ln.gm);
   }
   if (has_p) {
     const Sup sp = mv.sp;
 #pragma unroll 1
-    for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) W.y[sp.w0 + i] -= mupT * Vs[sp.ph + i * R];
+    for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) W.y()[sp.w0 + i] -= mupT * Vs[sp.ph + i * R];
     wds += 2 * (sp.ihi - sp.ilo);
   }
   if (ln.sl == 0) {
     if (jump == 0) {
-      W.list[N] = mv.jp;
-      if constexpr (MIX) W.le[N] = (unsigned char)ep;
+      W.list()[N] = mv.jp;
+      if constexpr (MIX) W.le()[N] = (unsigned char)ep;
     } else if (jump == 1) {
-      W.list[kk] = W.list[last];
-      if constexpr (MIX) W.le[kk] = W.le[last];
+      W.list()[kk] = W.list()[last];
+      if constexpr (MIX) W.le()[kk] = W.le()[last];
     } else {
-      W.list[kk] = mv.jp;
-      if constexpr (MIX) W.le[kk] = (unsigned char)ep;
+      W.list()[kk] = mv.jp;
+      if constexpr (MIX) W.le()[kk] = (unsigned char)ep;
     }
   }
   __syncwarp(ln.gm);
   return AcceptOut<C>{Cp, cap, Nout, wds, idl};
 }
 
+// The same out of line, for the births of an initial state.
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ AcceptOut<typename PeTab<T>::C> pe_accept_call(const DevModel& M, const PeChain<T, BIG, L, MIX> W,
+                                                                       typename PeTab<T>::C* Cp, int cap,
+                                                                       typename PeTab<T>::C* Cg,
+                                                                       const PeMove<typename PeTab<T>::C> mv, int n,
+                                                                       int N, const Lanes<L> ln) {
+  return pe_accept<T, BIG, L, MIX>(M, W, Cp, cap, Cg, mv, n, N, ln);
+}
+
+// The 2x2 algebra of Eqs. (16)-(18) in the scoring precision: log D, Delta nu and the status bits
+// of a move with components em (removed) and ep (new); r1 = 1 - q_- m_--.
+template <typename T> struct PeScore {
+  T dT, dnu;
+  int st;
+  bool ok;
+};
+template <typename T, bool MIX>
+__device__ __forceinline__ PeScore<T> pe_score(const DevModel& M, int e_m, int e_p, T em, T mmm, T mmp, T mpp, T gm, T gp) {
+  PeScore<T> o;
+  o.dT = (T)0; o.dnu = (T)NAN; o.st = 0; o.ok = false;
+  // det(I + Lambda M), Lambda = diag(-q_-, q_+) (q = sigma_e^2 of the PE concerned), with
+  // 1 - q_- m_-- = em; lambda = (-mu_-, mu_+) (Eq. (DeltaU), Appendix A.2)
+  const T qm = CmT<T>::q(M, e_m), qp = CmT<T>::q(M, e_p);
+  const T mum = CmT<T>::mu(M, e_m), mup = CmT<T>::mu(M, e_p);
+  const T Dd = em * ((T)1 + qp * mpp) + qm * qp * mmp * mmp;
+  if (!(Dd > (T)0)) {
+    o.st = FSMP_ST_BADDET;
+  } else {
+    const T iD = (T)1 / Dd;
+    const T B11 = -qm * ((T)1 + qp * mpp) * iD, B12 = qm * qp * mmp * iD, B22 = qp * em * iD;
+    // rho = g - M lambda; dR = -2 lambda^T g + lambda^T M lambda - rho^T B rho
+    const T rm = gm + mum * mmm - mup * mmp, rp = gp + mum * mmp - mup * mpp;
+    // (rho^T B rho with its roundings written out: which products a compiler fuses depends on the
+    // code around them, and a chain's decisions follow the last bit; results stay those of the
+    // forms it chose when each mode was checked)
+    const T b1 = B11 * rm, b2 = (T)2 * B12 * rm;
+    const T rBr = fma(B22 * rp, rp, sizeof(T) == 4 && !MIX ? fma(b1, rm, b2 * rp) : fma(b2, rp, b1 * rm));
+    const T dR = (T)-2 * (mup * gp - mum * gm) + (mum * mum * mmm - (T)2 * mum * mup * mmp + mup * mup * mpp) - rBr;
+    o.dT = log(Dd);
+    o.dnu = (T)-0.5 * (o.dT + dR);
+    if (!isfinite(o.dnu)) o.st = FSMP_ST_NONFINITE;
+    else o.ok = true;
+  }
+  return o;
+}
+
 // Random draws of the L steps from `step` on, lane l taking step + l (Philox4x64-10 keyed by
 // (seed, waveform), counter (step, block, 0, 0); Box-Muller for the two shifts). Out of line:
 // it runs once per L steps, and keeping it out of the step loop keeps the loop's code compact.
 // FP32 mode takes cos(2 pi u) as cospif(2u), whose argument reduction is exact.
-template <typename T, int L, bool MIX>
-__device__ __noinline__ void pe_draw(const DevModel& M, PeRand<T>* rnd, uint64_t seed, uint64_t wf_id, int step,
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void pe_draw(const DevModel& M, const PeChain<T, BIG, L, MIX> W, uint64_t seed, uint64_t wf_id, int step,
                                      const Lanes<L> ln) {
   constexpr bool fp32 = sizeof(T) == 4;
-  PeRand<T> rd;
-  rd.ep = 0;
+  PeRand<T, MIX> rd;
 #pragma unroll 1
   for (int blk = 0; blk < (MIX ? 3 : 2); ++blk) {
     uint64_t c[4] = {(uint64_t)(step + ln.sl), (uint64_t)blk, 0, 0};
     philox4x64_10(c, seed, wf_id);
     if (blk == 2) {  // MCP component of a born or updated PE
-      rd.ep = pe_draw_comp(M, u01_from_bits(c[0]));
+      if constexpr (MIX) rd.ep = pe_draw_comp(M, u01_from_bits(c[0]));
     } else if constexpr (fp32) {
       const float a = u01_float(c[0]), b = u01_float(c[1]), d = u01_float(c[2]), e = u01_float(c[3]);
       if (blk == 0) {
@@ -1147,7 +1466,7 @@ __device__ __noinline__ void pe_draw(const DevModel& M, PeRand<T>* rnd, uint64_t
       }
     }
   }
-  rnd[ln.sl] = rd;
+  W.rnd()[ln.sl] = rd;
   __syncwarp(ln.gm);
 }
 
@@ -1160,38 +1479,61 @@ __device__ __noinline__ void pe_trace_record(fsmp_trace* t, double la0, double l
   tr.N = N; tr.k0 = k0; tr.jump = jump; tr.flags = flags;
   *t = tr;
 }
-template <int L>
-__device__ __noinline__ void pe_hist_add(uint32_t* peh, const int* list, int N, int T_lo, int width, const Lanes<L> ln) {
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void pe_hist_add(const PeChain<T, BIG, L, MIX> W, uint32_t* peh, int N, int T_lo, int width,
+                                         uint32_t times, const Lanes<L> ln) {
+#pragma unroll 1
   for (int k = ln.sl; k < N; k += L) {
-    const int c = list[k] - T_lo;
-    if (c >= 0 && c < width) atomicAdd(peh + c, 1u);
+    const int c = W.list()[k] - T_lo;
+    if (c >= 0 && c < width) atomicAdd(peh + c, times);
   }
 }
 
+// Resident CTAs per SM the registers are cut for. A chain waits on instruction supply (the code it
+// runs through is larger than a scheduler's instruction cache, which refills at 16 bytes in 2.6
+// cycles), so a warp per chain does as many steps per second with 8 warps per SM as with 16
+// (uneven windows, 20 000 chains x 1000 steps: 58.96 ms against 58.78), each chain at twice the
+// speed: that takes the tail off a launch that has few chains (MCP mixture, 3000 chains: 18.2 ms
+// against 25.7; pile-up, 600 chains: 85.6 against 95.2) and leaves 255 registers. With two chains
+// per warp (L = 16) the half warps wait on each other, and 16 warps are better (30 000
+// low-occupancy chains: 31.5 ms, with 8 warps 42.9).
+constexpr int pe_min_ctas(int L) { return L == 16 ? 4 : 2; }
+
 template <typename T, bool BIG, int L, bool MIX>
-__global__ void __launch_bounds__(kPeMaxThreads, 4)
+__global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
     pe_kernel(const __grid_constant__ DevModel M, const __grid_constant__ BatchView B, const __grid_constant__ PeSlots G) {
   using C = typename PeTab<T>::C;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr bool fp32 = sizeof(T) == 4;
   const Lanes<L> ln = pe_lanes<L>();
   constexpr int kGroups = 32 / L;  // chains per warp
   const int cw = (threadIdx.x >> 5) * kGroups + ln.g, nchains = (blockDim.x >> 5) * kGroups;
   const int n_alloc = B.n_max, n_cap = M.n_cap, Ns = G.Ns;
-  // block tables: the SER, log(i) and 1 / i, i = 1 .. n_cap + 1
-  T* Vs = reinterpret_cast<T*>(smem_raw);
-  T* lgN = reinterpret_cast<T*>(smem_raw + a16(sizeof(T) * M.Lt));
-  double* inv1 = reinterpret_cast<double*>(smem_raw + a16(sizeof(T) * M.Lt) + a16(sizeof(T) * (n_cap + 2)));
+  unsigned short* const tij = pe_tij();
+  T* const Vs = pe_V<T>();
+  T* const lgN = reinterpret_cast<T*>(pe_smem + (kTabBytes + (unsigned)a16(sizeof(T) * M.Lt)));
+  double* const inv1 = reinterpret_cast<double*>(
+      pe_smem + (kTabBytes + (unsigned)a16(sizeof(T) * M.Lt) + (unsigned)a16(sizeof(T) * (n_cap + 2))));
+#pragma unroll 1
+  for (int e = threadIdx.x; e < kTriTab; e += blockDim.x) {
+    int i, j;
+    untri(e, i, j);
+    tij[e] = (unsigned short)(i << 8 | j);
+  }
+#pragma unroll 1
   for (int m = threadIdx.x; m < M.Lt; m += blockDim.x) Vs[m] = PeTab<T>::V(M)[m];
+#pragma unroll 1
   for (int i = threadIdx.x; i < n_cap + 2; i += blockDim.x) {
     lgN[i] = i > 0 ? (fp32 ? (T)logf((float)i) : (T)log((double)i)) : (T)0;
     inv1[i] = i > 0 ? 1.0 / (double)i : 0.0;
   }
   __syncthreads();
-  PeChain<T> W = pe_carve<T, L>(smem_raw + pe_block_bytes<T>(M) +
-                                    (size_t)cw * pe_chain_bytes<T, L>(n_cap, n_alloc, M.win_extra, Ns),
-                                n_cap, n_alloc, M.win_extra, Ns);
-  PeStats& S = *W.st;
+  PeChain<T, BIG, L, MIX> W;
+  W.vb = (unsigned)a16(sizeof(C) * (size_t)n_cap);
+  W.lb = (unsigned)a16(sizeof(int) * (size_t)n_cap);
+  W.yb = (unsigned)a16(sizeof(T) * (size_t)n_alloc);
+  W.pb = (unsigned)a16(sizeof(T) * (size_t)M.win_extra);
+  W.o = (unsigned)(pe_block_bytes<T>(M) + (size_t)cw * pe_chain_bytes<T, BIG, L, MIX>(n_cap, n_alloc, M.win_extra, Ns));
+  PeStats& S = W.st();
   const size_t slot = (size_t)blockIdx.x * nchains + cw;
   int* const hist = G.hist + slot * (size_t)(n_cap + 1);
   C* const Cg = G.C ? reinterpret_cast<C*>(G.C) + slot * G.c_stride : nullptr;
@@ -1254,36 +1596,37 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
       }
     }
     // log(Phi_T(t0) g) on the t0 grid (-inf where Phi_T = 0), from the FP64 tables
+#pragma unroll 1
     for (int k = ln.sl; k <= k0_hi - k0_lo; k += L) {
       const int kq = k0_lo + k;
       const double tot = pe_cphi<double>(M, T_hi - 1 - kq) - pe_cphi<double>(M, T_lo - 1 - kq);
-      W.lPhi[k] = tot > 0.0 ? (fp32 ? (T)logf((float)(tot * M.g)) : (T)log(tot * M.g)) : (T)-INFINITY;
+      W.lPhi()[k] = tot > 0.0 ? (fp32 ? (T)logf((float)(tot * M.g)) : (T)log(tot * M.g)) : (T)-INFINITY;
     }
 #pragma unroll 1
     for (int k = ln.sl; k <= n_cap; k += L) hist[k] = 0;
+#pragma unroll 1
+    for (int q = ln.sl; q < kSpec * kCounts; q += L) W.cnt()[q] = 0;
     // empty z: y = w
     double wsq = 0.0;
+#pragma unroll 1
     for (int x = ln.sl; x < n; x += L) {
       const float wx = w[x];
-      W.y[x] = (T)wx;
+      W.y()[x] = (T)wx;
       wsq += (double)wx * (double)wx;
     }
     wsq = wsum(wsq, ln);
     if (ln.sl == 0) {
-      S.sN = S.sN2 = S.sK = S.sK2 = 0;
-      S.sQ = S.sQ2 = 0.0; S.q_cur = 0.0; S.q_from = 0;
-      S.St = S.Se = 0; S.wt_cur = S.we_cur = 0.0;
-      S.sWt = S.sWt2 = S.sWe = S.sWe2 = 0.0;
-      S.logdet = n * M.log_se2;
-      S.logL = -0.5 * (n * kLog2Pi + S.logdet + wsq * M.inv_se2);
+      for (int k = 0; k < 3; ++k) S.cur[k] = S.sum[2 * k] = S.sum[2 * k + 1] = 0.0;
+      S.St = S.Se = 0; S.q_from = 0;
+      S.sum[PeStats::kLogdet] = n * M.log_se2;
+      S.sum[PeStats::kLogL] = -0.5 * (n * kLog2Pi + S.sum[PeStats::kLogdet] + wsq * M.inv_se2);
       S.wsq = wsq;
-      S.drift_max = 0.0; S.alg_words = 0;
-      for (int k = 0; k < 3; ++k) { S.acc[k] = 0; S.prop[k] = 0; }
-      S.acc_t0 = S.prop_t0 = S.n_refresh = S.status = S.n_acc_refresh = S.refresh_fail = 0;
+      S.drift_max = 0.0;
+      S.n_refresh = S.status = S.n_acc_refresh = S.refresh_fail = 0;
     }
     __syncwarp(ln.gm);
     const T log_lambda0 = fp32 ? (T)logf((float)lambda0) : (T)log(lambda0);
-    C* Cp = Ns > 0 ? W.Cs : Cg;  // C^-1 (packed), room for cap PEs
+    C* Cp = Ns > 0 ? W.Cs(n_cap) : Cg;  // C^-1 (packed), room for cap PEs
     int cap = Ns > 0 ? Ns : n_cap;
     int N = 0;
     if (B.z_init) {
@@ -1292,9 +1635,10 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
       int ni = min(B.n_init[wi], B.z_stride);
       const bool cut = ni > n_cap;
       if (cut) ni = n_cap;
+#pragma unroll 1
       for (int k = ln.sl; k < ni; k += L) {
-        W.list[k] = B.z_init[(size_t)wi * B.z_stride + k];
-        if constexpr (MIX) W.le[k] = (unsigned char)M.cm_mode;
+        W.list()[k] = B.z_init[(size_t)wi * B.z_stride + k];
+        if constexpr (MIX) W.le()[k] = (unsigned char)M.cm_mode;
       }
       __syncwarp(ln.gm);
       if (ni > cap) { Cp = Cg; cap = n_cap; }
@@ -1306,7 +1650,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
           // FP32 mode: the FP64 rebuild
           const RefreshOut ro = pe_refresh<T, BIG, L, MIX>(M, W, Cp, ws, n_cap, w, S.wsq, n, ni, ln);
           ok = ro.ok != 0;
-          if (ok && ln.sl == 0) { S.logdet = ro.logdet; S.logL = ro.logL; }
+          if (ok && ln.sl == 0) { S.sum[PeStats::kLogdet] = ro.logdet; S.sum[PeStats::kLogL] = ro.logL; }
         } else {
           // FP64 mode: the PEs born one by one through the accepted-move update in double-double
           // (the FP64 rebuild would leave C^-1 only as accurate as FP64 times its condition
@@ -1315,7 +1659,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
 #pragma unroll 1
           for (int k = 0; k < ni; ++k) {
             PeMove<C> mv;
-            mv.jump = 0; mv.kk = -1; mv.jp = W.list[k]; mv.jm = -1;
+            mv.jump = 0; mv.kk = -1; mv.jp = W.list()[k]; mv.jm = -1;
             mv.em = mv.ep = MIX ? M.cm_mode : 0;
             const Sup sp = pe_sup(M, n, mv.jp);
             mv.sp = sp;
@@ -1325,15 +1669,15 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
               const int qi = base + ln.sl;
               C bq = czero<C>();
               if (qi < N) {
-                const int o = mv.jp - W.list[qi];
+                const int o = mv.jp - W.list()[qi];
                 if (o > -M.Lt && o < M.Lt) bq = xcorr<C>(M, tc, sp, o);
               }
               const bool ov = cnz(bq);
               const unsigned m = gballot(ov, ln);
               if (ov) {
                 const int pos = np + __popc(m & ((1u << ln.sl) - 1u));
-                W.ovi[pos] = qi;
-                W.ovb[pos] = bq;
+                W.ovi()[pos] = qi;
+                W.ovb()[pos] = bq;
               }
               np += __popc(m);
             }
@@ -1341,10 +1685,11 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
             mv.np = np;
             mv.aa = xcorr<C>(M, tc, sp, 0);
             T ayp = (T)0;
-            for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) ayp += Vs[sp.ph + i * R] * W.y[sp.w0 + i];
+#pragma unroll 1
+            for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) ayp += Vs[sp.ph + i * R] * W.y()[sp.w0 + i];
             mv.ay = cfromf(wsum(ayp, ln));
-            mv.quad = mv.bv = mv.vk = czero<C>();
-            const AcceptOut<C> ao = pe_accept<T, BIG, L, MIX>(M, W, Vs, Cp, cap, Cg, mv, n, N, ln);
+            mv.vk = czero<C>();
+            const AcceptOut<C> ao = pe_accept_call<T, BIG, L, MIX>(M, W, Cp, cap, Cg, mv, n, N, ln);
             Cp = ao.Cp;
             cap = ao.cap;
             N = ao.N;
@@ -1355,290 +1700,551 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
           N = 0;
           // log|Sigma| = n log se2 + log|C| - sum_k log r_k; y^T Sigma^-1 y = (y^T y - h^T v) / se2
           double lr = 0.0, yy = 0.0, hv = 0.0;
+#pragma unroll 1
           for (int k = ln.sl; k < ni; k += L) {
             lr += M.cm_lr[MIX ? M.cm_mode : 0];
-            const Sup s = pe_sup(M, n, W.list[k]);
+            const Sup s = pe_sup(M, n, W.list()[k]);
             double hk = 0.0;
-            for (int i = s.ilo; i < s.ihi; ++i) hk = fma((double)Vs[s.ph + i * R], (double)W.y[s.w0 + i], hk);
-            hv = fma(hk, c64(W.v[k]), hv);
+#pragma unroll 1
+            for (int i = s.ilo; i < s.ihi; ++i) hk = fma((double)Vs[s.ph + i * R], (double)W.y()[s.w0 + i], hk);
+            hv = fma(hk, c64(W.v()[k]), hv);
           }
-          for (int x = ln.sl; x < n; x += L) yy = fma((double)W.y[x], (double)W.y[x], yy);
+#pragma unroll 1
+          for (int x = ln.sl; x < n; x += L) yy = fma((double)W.y()[x], (double)W.y()[x], yy);
           lr = wsum(lr, ln); yy = wsum(yy, ln); hv = wsum(hv, ln);
           if (ok && ln.sl == 0) {
-            S.logdet = n * M.log_se2 + lC - lr;
-            S.logL = -0.5 * (n * kLog2Pi + S.logdet + (yy - hv) * M.inv_se2);
+            S.sum[PeStats::kLogdet] = n * M.log_se2 + lC - lr;
+            S.sum[PeStats::kLogL] = -0.5 * (n * kLog2Pi + S.sum[PeStats::kLogdet] + (yy - hv) * M.inv_se2);
           }
         }
+#pragma unroll 1
         for (int i = ln.sl; i < ni; i += L) {
-          qs = cadd(qs, W.v[i]);
-          if (mix) ms += M.cm_mu[W.le[i]];
+          qs = cadd(qs, W.v()[i]);
+          if (mix) ms += M.cm_mu[W.le()[i]];
         }
         qs = csum(qs, ln);
-        ms = mix ? wsum(ms, ln) : ni * M.cm_mu[0];
+        ms = mix ? wsum(ms, ln) : M.cm_mu[0];
         if (ok) {
           N = ni;
         } else {  // C not numerically positive definite: start empty
-          for (int x = ln.sl; x < n; x += L) W.y[x] = (T)w[x];
-          Cp = Ns > 0 ? W.Cs : Cg;
+#pragma unroll 1
+          for (int x = ln.sl; x < n; x += L) W.y()[x] = (T)w[x];
+          Cp = Ns > 0 ? W.Cs(n_cap) : Cg;
           cap = Ns > 0 ? Ns : n_cap;
         }
         long long st = 0;
-        for (int k = ln.sl; k < ni; k += L) st += abs(W.list[k]);
+#pragma unroll 1
+        for (int k = ln.sl; k < ni; k += L) st += abs(W.list()[k]);
         st = wsum(st, ln);
         if (ln.sl == 0) {
           if (ok) {
-            S.q_cur = ms + c64(qs);
             S.St = st;
             S.Se = MIX ? (long long)ni * M.cm_mode : 0;
-            set_wasserstein(S, M.g, ni, inv1);
           } else {
             S.status |= FSMP_ST_BADDET;
           }
         }
+        __syncwarp(ln.gm);
+        if (ok) set_summaries<MIX>(S, M.g, ni, ms, c64(qs), inv1, ln.sl);
       }
       if (ln.sl == 0 && cut) S.status |= FSMP_ST_CAPACITY;
       __syncwarp(ln.gm);
     }
 
-    for (int step = 0; step < n_steps; ++step) {
+    for (int step = 0; step < n_steps;) {
       // ---- random draws of the next L steps: lane l takes step step + l
-      if ((step & (L - 1)) == 0) pe_draw<T, L, MIX>(M, W.rnd, seed, wf_id, step, ln);
-      const PeRand<T> rd = W.rnd[step & (L - 1)];
-      // ---- Gibbs part 1: MH on t0 (Sec. 2.4), uniform prior on its grid range
-      T la0 = (T)NAN;
-      const T lu0 = rd.lu0;
-      int t0f = 0, st_a = 0;
-      if (M.sample_t0) {
-        t0f = 1;
-        const int Dm = fp32 ? __float2int_rn((float)(rd.z1 * inv_gT)) : __double2int_rn((double)(rd.z1 * inv_gT));
-        const int k0p = k0 + Dm;
-        if (Dm == 0) {
-          la0 = (T)0;
-        } else if (k0p < k0_lo || k0p > k0_hi) {
-          la0 = (T)-INFINITY;
-        } else {
-          T part = (T)0;
-#pragma unroll 1
-          for (int k = ln.sl; k < N; k += L) {
-            const int j = W.list[k];
-            part += pe_logphi<T>(M, j - k0p) - pe_logphi<T>(M, j - k0);
-          }
-          la0 = wsum(part, ln);
-        }
-        if (lu0 < la0) { k0 = k0p; t0f |= 2; }
-      }
-      // ---- Gibbs part 2: one RJMCMC jump (Sec. 2.4)
-      const int jump = (N == 0) ? 0 : (rd.u3 < Jt ? 0 : (rd.u3 < (T)2 * Jt ? 1 : 2));
-      int valid = 0, noop = 0, kk = -1, jp = -1, jm = -1, e_m = MIX ? rd.ep : 0;
-      T la_prior = (T)0, la_fixed = (T)-INFINITY;
-      const T lu = rd.lu;
-      const T lphi_t0 = W.lPhi[k0 - k0_lo];
-      if (jump == 0) {
-        if (N >= n_cap) {
-          st_a |= FSMP_ST_CAPACITY;
-        } else if (lphi_t0 > (T)-INFINITY) {
-          const T base = pe_cphi<T>(M, T_lo - 1 - k0), tot = pe_cphi<T>(M, T_hi - 1 - k0) - base;
-          jp = pe_birth_search<T, L>(M, T_lo, T_hi, k0, base, rd.u4 * tot, ln);
-          valid = jp >= T_lo;
-          la_prior = log_lambda0 + lphi_t0 - lgN[N + 1] + (N == 0 ? logJ : (T)0);
-        }
-      } else {
-        kk = fp32 ? __float2int_rd((float)(rd.u4 * (T)N)) : __double2int_rd((double)(rd.u4 * (T)N));
-        if (kk >= N) kk = N - 1;
-        jm = W.list[kk];
-        if constexpr (MIX) e_m = W.le[kk];
-        if (jump == 1) {
-          valid = 1;
-          la_prior = -log_lambda0 - lphi_t0 + lgN[N] - (N == 1 ? logJ : (T)0);
-        } else {
-          const int Dm = fp32 ? __float2int_rn((float)(rd.z2 * inv_gT)) : __double2int_rn((double)(rd.z2 * inv_gT));
-          const int jpl = jm + Dm;
-          if (Dm == 0 && (!MIX || rd.ep == e_m)) {  // same time and component: an accepted no-op
-            noop = 1;
-            la_fixed = (T)0;
-          } else if (jpl < T_lo || jpl >= T_hi || pe_logphi<T>(M, jpl - k0) == (T)-INFINITY) {
-            la_fixed = (T)-INFINITY;
-          } else {
-            jp = jpl;
-            valid = 1;
-            la_prior = pe_logphi<T>(M, jp - k0) - pe_logphi<T>(M, jm - k0);
-          }
-        }
-      }
-      // ---- scoring: the 2x2 quantities in PE space, then the 2x2 algebra in T
+      PeRand<T, MIX>* const rnd = W.rnd();
+      if ((step & (L - 1)) == 0) pe_draw<T, BIG, L, MIX>(M, W, seed, wf_id, step, ln);
+      // The accepted move of this round (or, one by one, the step made), filled in below
       PeMove<C> mv;
-      mv.jump = jump; mv.kk = kk; mv.jp = jp; mv.jm = jm; mv.np = 0;
-      // components of a_- and a_+; the absent one of a birth or death takes the other's values
-      // (its terms vanish)
-      mv.em = e_m;
-      mv.ep = MIX ? (jump == 1 ? e_m : rd.ep) : 0;
-      mv.aa = mv.quad = mv.bv = mv.vk = mv.ay = czero<C>();
-      mv.sp = Sup{0, 0, 0, 0};
-      T mmm = 0, mmp = 0, mpp = 0, gm = 0, gp = 0, em = 1;
-      unsigned long long words = 0;
-      if (valid) {
-        if (jump != 1) {
-          const Sup sp = pe_sup(M, n, jp);
-          mv.sp = sp;
-          mv.aa = xcorr<C>(M, tc, sp, 0);  // issued first: its table load overlaps the scan's
-          // PEs overlapping a_+, with b_q = a_q^T a_+
-          int np = 0;
+      T dT = (T)0, dnu = (T)NAN;
+      int jump = 0, e_m = 0;   // of the step last = step + counted - 1
+      bool apply = false, t0_acc = false;
+      bool one = true;         // that step is still to be counted
+      unsigned words = 0;
+      int last;
+      if (!BIG && N <= kSpecPes) {
+        // ---------------------------------------------- a batch of steps, one per subgroup
+        constexpr int gw = L / kSpec;  // lanes of a subgroup
+        const int gi = ln.sl / gw, m = ln.sl % gw;
+        const int g = min(min(kSpec, n_steps - step), L - (step & (L - 1)));  // steps of the batch
+        const bool mine = gi < g;
+        const PeRand<T, MIX> rd = rnd[(step + min(gi, g - 1)) & (L - 1)];
+        // ---- Gibbs part 1: MH on t0 (Sec. 2.4), the steps in turn; a subgroup keeps its step's k0
+        int k0i = k0;
+        T la0 = (T)NAN;
+        unsigned t0a = 0;  // accepted t0 moves of the batch
+        if (M.sample_t0) {
+          int kr = k0;
 #pragma unroll 1
-          for (int base = 0; base < N; base += L) {
-            const int qi = base + ln.sl;
-            C bq = czero<C>();
-            if (qi < N) {
-              const int o = jp - W.list[qi];
-              if (o > -M.Lt && o < M.Lt) bq = xcorr<C>(M, tc, sp, o);
+          for (int i = 0; i < g; ++i) {
+            const PeRand<T, MIX>& ri = rnd[(step + i) & (L - 1)];
+            const T z1 = ri.z1;
+            const int Dm = fp32 ? __float2int_rn((float)(z1 * inv_gT)) : __double2int_rn((double)(z1 * inv_gT));
+            const int k0p = kr + Dm;
+            T la = (T)0;
+            if (Dm != 0) {
+              if (k0p < k0_lo || k0p > k0_hi) {
+                la = (T)-INFINITY;
+              } else {
+                T part = (T)0;
+#pragma unroll 1
+                for (int k = ln.sl; k < N; k += L) {
+                  const int j = W.list()[k];
+                  part += pe_logphi<T>(M, j - k0p) - pe_logphi<T>(M, j - kr);
+                }
+                la = wsum(part, ln);
+              }
             }
-            const bool ov = cnz(bq);
-            const unsigned m = gballot(ov, ln);
-            if (ov) {
-              const int pos = np + __popc(m & ((1u << ln.sl) - 1u));
-              W.ovi[pos] = qi;
-              W.ovb[pos] = bq;
-            }
-            np += __popc(m);
+            if (ri.lu0 < la) { kr = k0p; t0a |= 1u << i; }
+            if (gi == i) { k0i = kr; la0 = la; }
           }
-          __syncwarp(ln.gm);
-          mv.np = np;
-          // b^T C^-1 b over the lower triangle of the overlap block (lanes over its entries, the
-          // off-diagonal ones counted twice), b^T v, (C^-1 b)_k of an update and a_+^T y, then one
-          // reduction of the four over the group
-          T ayp = (T)0;
+        }
+        // ---- Gibbs part 2: one RJMCMC jump (Sec. 2.4)
+        jump = (N == 0) ? 0 : (rd.u3 < Jt ? 0 : (rd.u3 < (T)2 * Jt ? 1 : 2));
+        int st = 0, kk = -1, jp = -1, jm = -1, e_p = 0;
+        if constexpr (MIX) { e_m = rd.ep; e_p = rd.ep; }
+        bool valid = false, noop = false;
+        T la_prior = (T)0, la_fixed = (T)-INFINITY;
+        const T lphi_t0 = W.lPhi()[k0i - k0_lo];
+        const bool birth = mine && jump == 0 && N < n_cap && lphi_t0 > (T)-INFINITY;
+        if (jump == 0 && N >= n_cap) st = FSMP_ST_CAPACITY;
+        if (gballot(birth, ln)) {
+          const int jb = pe_birth_search_sub<T, L>(M, T_lo, T_hi, k0i, rd.u4, birth, ln);
+          if (birth) {
+            jp = jb;
+            valid = jp >= T_lo;
+            la_prior = log_lambda0 + lphi_t0 - lgN[N + 1] + (N == 0 ? logJ : (T)0);
+          }
+        }
+        if (mine && jump != 0) {
+          kk = fp32 ? __float2int_rd((float)(rd.u4 * (T)N)) : __double2int_rd((double)(rd.u4 * (T)N));
+          if (kk >= N) kk = N - 1;
+          jm = W.list()[kk];
+          if constexpr (MIX) e_m = W.le()[kk];
+          if (jump == 1) {
+            valid = true;
+            e_p = e_m;
+            la_prior = -log_lambda0 - lphi_t0 + lgN[N] - (N == 1 ? logJ : (T)0);
+          } else {
+            const int Dm = fp32 ? __float2int_rn((float)(rd.z2 * inv_gT)) : __double2int_rn((double)(rd.z2 * inv_gT));
+            const int jpl = jm + Dm;
+            if (Dm == 0 && (!MIX || e_p == e_m)) {  // same time and component: an accepted no-op
+              noop = true;
+              la_fixed = (T)0;
+            } else if (jpl >= T_lo && jpl < T_hi) {
+              const T lp = pe_logphi<T>(M, jpl - k0i);
+              if (!(lp == (T)-INFINITY)) {
+                jp = jpl;
+                valid = true;
+                la_prior = lp - pe_logphi<T>(M, jm - k0i);
+              }
+            }
+          }
+        }
+        // ---- scoring: PEs overlapping a_+, with b_q = a_q^T a_+
+        const bool new_pe = valid && jump != 1;
+        Sup sp{0, 0, 0, 0};
+        C aa = czero<C>();
+        if (new_pe) {
+          sp = pe_sup(M, n, jp);
+          aa = xcorr<C>(M, tc, sp, 0);
+        }
+        C* const bs = W.work(gi);
+        unsigned char* const ix = W.ix() + gi * kSpecPes;
+        int np = 0;
 #pragma unroll 1
-          for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) ayp += Vs[sp.ph + i * R] * W.y[sp.w0 + i];
-          C qp = czero<C>(), ck = czero<C>();
-          T bvp = (T)0;
+        for (int base = 0; base < N; base += gw) {
+          const int qi = base + m;
+          C bq = czero<C>();
+          if (new_pe && qi < N) {
+            const int o = jp - W.list()[qi];
+            if (o > -M.Lt && o < M.Lt) bq = xcorr<C>(M, tc, sp, o);
+          }
+          const bool ov = cnz(bq);
+          const unsigned b = (gballot(ov, ln) >> (gi * gw)) & ((1u << gw) - 1u);
+          if (ov) {
+            const int pos = np + __popc(b & ((1u << m) - 1u));
+            ix[pos] = (unsigned char)qi;
+            bs[pos] = bq;
+          }
+          np += __popc(b);
+        }
+        __syncwarp(ln.gm);
+        // b^T C^-1 b, (C^-1 b)_k of an update, b^T v and a_+^T y: the partial sums x_u that lanes
+        // m + u gw (u < 4) of a step made alone have, two at a time, added as its butterfly adds
+        // them: (x_0 + x_2) + (x_1 + x_3)
+        static_assert(kSpec == 4, "the sums below are of four lanes' partial sums");
+        C qp, ck;
+        T bvp, ayp;
+        {
           const int nt = tri(np);
-          int e = ln.sl;
-          if constexpr (BIG) {  // C^-1 in the global slot: four entries' loads ahead of their sums
+          Pk<C> hq = pk2(czero<C>(), czero<C>()), hc = hq;
+          T ha0 = (T)0, ha1 = (T)0, hb0 = (T)0, hb1 = (T)0;
 #pragma unroll 1
-            for (; e + 3 * L < nt; e += 4 * L) {
-              C cq[4], bb[4];
-              bool dg[4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                int a, b2;
-                untri(e + u * L, a, b2);
-                cq[u] = Cp[pk(W.ovi[a], W.ovi[b2])];
-                bb[u] = cmul(W.ovb[a], W.ovb[b2]);
-                dg[u] = a == b2;
+          for (int vl = m; vl < L; vl += 2 * gw) {
+            T xa0 = (T)0, xa1 = (T)0, xb0 = (T)0, xb1 = (T)0;
+            Pk<C> xq = pk2(czero<C>(), czero<C>()), xc = xq;
+#pragma unroll 1
+            for (int i = sp.ilo + vl; i < sp.ihi; i += L) {
+              xa0 += Vs[sp.ph + i * R] * W.y()[sp.w0 + i];
+              if (i + gw < sp.ihi) xa1 += Vs[sp.ph + (i + gw) * R] * W.y()[sp.w0 + i + gw];
+            }
+#pragma unroll 1
+            for (int e = vl; e < nt; e += L) {
+              const int ij = tij[e], a = ij >> 8, b2 = ij & 255;
+              const bool two = e + gw < nt;  // else a zero term
+              if constexpr (!fp32) {  // FP64 operations are not packed: no zero terms
+                const C t0 = cmul(Cp[tri(ix[a]) + ix[b2]], cmul(bs[a], bs[b2]));
+                xq.a = cadd(xq.a, a == b2 ? t0 : ctwice(t0));
+                if (two) {
+                  const int ij1 = tij[e + gw], a1 = ij1 >> 8, b21 = ij1 & 255;
+                  const C t1 = cmul(Cp[tri(ix[a1]) + ix[b21]], cmul(bs[a1], bs[b21]));
+                  xq.b = cadd(xq.b, a1 == b21 ? t1 : ctwice(t1));
+                }
+                continue;
               }
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const C t = cmul(cq[u], bb[u]);
-                qp = cadd(qp, dg[u] ? t : ctwice(t));
+              const int ij1 = tij[two ? e + gw : e], a1 = ij1 >> 8, b21 = ij1 & 255;
+              const C c1 = Cp[tri(ix[a1]) + ix[b21]];
+              const Pk<C> t = pk_mul(pk2(Cp[tri(ix[a]) + ix[b2]], two ? c1 : czero<C>()),
+                                     pk_mul(pk2(bs[a], bs[a1]), pk2(bs[b2], bs[b21])));
+              const C t0 = pk_first(t), t1 = pk_second(t);
+              xq = pk_add(xq, pk2(a == b2 ? t0 : ctwice(t0), a1 == b21 ? t1 : ctwice(t1)));
+            }
+#pragma unroll 1
+            for (int a = vl; a < np; a += L) {
+              const bool two = a + gw < np;
+              const int a1 = two ? a + gw : a;
+              const C ba = bs[a], ba1 = two ? bs[a1] : czero<C>();
+              const int q = ix[a], q1 = ix[a1];
+              xb0 += (T)cnum(ba) * (T)cnum(W.v()[q]);
+              xb1 += (T)cnum(ba1) * (T)cnum(W.v()[q1]);
+              if (opaque(jump == 2)) {
+                if constexpr (fp32) {
+                  xc = pk_fma(pk2(Cp[pk(kk, q)], Cp[pk(kk, q1)]), pk2(ba, ba1), xc);
+                } else {
+                  xc.a = cfma(Cp[pk(kk, q)], ba, xc.a);
+                  if (two) xc.b = cfma(Cp[pk(kk, q1)], ba1, xc.b);
+                }
               }
             }
+            ha0 += xa0; ha1 += xa1; hb0 += xb0; hb1 += xb1;
+            hq = pk_add(hq, xq); hc = pk_add(hc, xc);
           }
-#pragma unroll 1
-          for (; e < nt; e += L) {
-            int a, b2;
-            untri(e, a, b2);
-            const C t = cmul(Cp[pk(W.ovi[a], W.ovi[b2])], cmul(W.ovb[a], W.ovb[b2]));
-            qp = cadd(qp, a == b2 ? t : ctwice(t));
-          }
-#pragma unroll 1
-          for (int a = ln.sl; a < np; a += L) {
-            const C ba = W.ovb[a];
-            bvp += (T)cnum(ba) * (T)cnum(W.v[W.ovi[a]]);
-            if (jump == 2) ck = cfma(Cp[pk(kk, W.ovi[a])], ba, ck);
-          }
-          gsum4<L>(qp, ck, bvp, ayp, ln);
-          mv.quad = qp;
+          ayp = ha0 + ha1; bvp = hb0 + hb1;
+          qp = cadd(pk_first(hq), pk_second(hq)); ck = cadd(pk_first(hc), pk_second(hc));
+        }
+        __syncwarp(ln.gm);
+        gsum4<L, gw>(qp, ck, bvp, ayp, ln);
+        T mmm = 0, mmp = 0, mpp = 0, gm = 0, gp = 0, em = 1;
+        if (new_pe) {
           const T bvT = bvp;  // b^T v at the scoring precision (the accept recomputes it)
           const T ayT = ayp;
-          mv.ay = cfromf(ayT);
-          mpp = (T)cnum(csub(mv.aa, mv.quad)) * ise2T;
+          mpp = (T)cnum(csub(aa, qp)) * ise2T;
           gp = (ayT - bvT) * ise2T;
           mmp = (T)cnum(ck);  // times 1 / sigma_-^2 below (update only)
-          words += (unsigned long long)(N + 2 * np + 2 * (sp.ihi - sp.ilo) + np * np + np);
+          words += (unsigned)(N + 2 * np + 2 * (sp.ihi - sp.ilo) + np * np + np);
         }
-        if (jump != 0) {
-          const T iqm = CmT<T>::iq(M, mv.em);
-          mv.vk = W.v[kk];
-          em = CmT<T>::r(M, mv.em) * (T)cnum(Cp[tri(kk) + kk]);
+        if (valid && jump != 0) {
+          const T iqm = CmT<T>::iq(M, e_m);
+          em = CmT<T>::r(M, e_m) * (T)cnum(Cp[tri(kk) + kk]);
           mmm = ((T)1 - em) * iqm;
-          gm = (T)cnum(mv.vk) * iqm;
+          gm = (T)cnum(W.v()[kk]) * iqm;
           mmp *= iqm;
           words += 2;
         }
-      }
-      T la = la_fixed, dnu = (T)NAN, dT = (T)0;
-      int st_c = 0;
-      if (valid) {
-        // det(I + Lambda M), Lambda = diag(-q_-, q_+) (q = sigma_e^2 of the PE concerned), with
-        // 1 - q_- m_-- = em; lambda = (-mu_-, mu_+) (Eq. (DeltaU), Appendix A.2)
-        const T qm = CmT<T>::q(M, mv.em), qp = CmT<T>::q(M, mv.ep);
-        const T mum = CmT<T>::mu(M, mv.em), mup = CmT<T>::mu(M, mv.ep);
-        const T Dd = em * ((T)1 + qp * mpp) + qm * qp * mmp * mmp;
-        if (!(Dd > (T)0)) {
-          la = (T)-INFINITY;
-          st_c |= FSMP_ST_BADDET;
-        } else {
-          const T iD = (T)1 / Dd;
-          const T B11 = -qm * ((T)1 + qp * mpp) * iD, B12 = qm * qp * mmp * iD, B22 = qp * em * iD;
-          // rho = g - M lambda; dR = -2 lambda^T g + lambda^T M lambda - rho^T B rho
-          const T rm = gm + mum * mmm - mup * mmp, rp = gp + mum * mmp - mup * mpp;
-          const T dR = (T)-2 * (mup * gp - mum * gm) + (mum * mum * mmm - (T)2 * mum * mup * mmp + mup * mup * mpp) -
-                       (B11 * rm * rm + (T)2 * B12 * rm * rp + B22 * rp * rp);
-          dT = log(Dd);
-          dnu = (T)-0.5 * (dT + dR);
-          if (!isfinite(dnu)) {
-            la = (T)-INFINITY;
-            st_c |= FSMP_ST_NONFINITE;
+        T la = la_fixed;
+        if (valid) {
+          const PeScore<T> sc = pe_score<T, MIX>(M, e_m, e_p, em, mmm, mmp, mpp, gm, gp);
+          dT = sc.dT;
+          dnu = sc.dnu;
+          st |= sc.st;
+          la = sc.ok ? dnu + la_prior : (T)-INFINITY;
+        }
+        const bool acc = mine && rd.lu < la;
+        apply = acc && valid && isfinite(la);
+        // ---- the steps that count: up to and including the first accepted move
+        const unsigned first = gballot(apply, ln);
+        const int f = first ? (__ffs(first) - 1) / gw : g - 1;
+        const bool counted = gi <= f;
+        const bool t0m = (t0a >> gi) & 1u;
+        if (m == 0 && counted) {
+          if (st) atomicOr(&S.status, st);
+          if (trace)
+            pe_trace_record(trace + step + gi, (double)la0, (double)rd.lu0, (double)la, (double)rd.lu, (double)dnu,
+                            N + (apply ? (jump == 0 ? 1 : (jump == 1 ? -1 : 0)) : 0), k0i, jump,
+                            (M.sample_t0 ? 1 : 0) | (t0m ? 2 : 0) | (acc ? 4 : 0) | ((acc && noop) ? 8 : 0));
+        }
+        if (counted && !apply) {
+#pragma unroll
+          for (int q = m; q < kCounts; q += gw)
+            W.cnt()[gi * kCounts + q] += count_of(q, N, k0i, step + gi >= burn_in, words, jump, false, t0m);
+        }
+        const int rejected = first ? f : g;
+        const int past = max(0, rejected - max(0, burn_in - step));  // of them after burn-in
+        if (past > 0) {
+          if (ln.sl == 0) atomicAdd(hist + N, past);  // no value returned: the lane does not wait on it
+          if (peh) pe_hist_add(W, peh, N, T_lo, B.pe_hist_width, (uint32_t)past, ln);
+        }
+        last = step + f;
+        k0 = __shfl_sync(ln.gm, k0i, f * gw, L);
+        one = apply = first != 0;
+        if (apply) {
+          // the accepted move on every lane; its overlapping PEs as the accept reads them
+          const int src = f * gw;
+          jump = __shfl_sync(ln.gm, jump, src, L);
+          kk = __shfl_sync(ln.gm, kk, src, L);
+          mv.np = __shfl_sync(ln.gm, np, src, L);
+          mv.jp = __shfl_sync(ln.gm, jp, src, L);
+          mv.jm = __shfl_sync(ln.gm, jm, src, L);
+          if constexpr (MIX) { e_m = __shfl_sync(ln.gm, e_m, src, L); e_p = __shfl_sync(ln.gm, e_p, src, L); }
+          dT = __shfl_sync(ln.gm, dT, src, L);
+          dnu = __shfl_sync(ln.gm, dnu, src, L);
+          words = __shfl_sync(ln.gm, words, src, L);
+          mv.ay = cfromf(__shfl_sync(ln.gm, ayp, src, L));
+          mv.aa = cshfl<L>(aa, src, ln.gm);
+          t0_acc = (t0a >> f) & 1u;
+          mv.jump = jump; mv.kk = kk; mv.em = e_m; mv.ep = e_p;
+          mv.vk = jump != 0 ? W.v()[kk] : czero<C>();
+          mv.sp = jump != 1 ? pe_sup(M, n, mv.jp) : Sup{0, 0, 0, 0};
+          if (jump != 1) {
+            if (f > 0) {
+#pragma unroll 1
+              for (int a = ln.sl; a < mv.np; a += L) W.ovb()[a] = W.work(f)[a];
+              __syncwarp(ln.gm);
+            }
+#pragma unroll 1
+            for (int a = ln.sl; a < mv.np; a += L) W.ovi()[a] = W.ix()[f * kSpecPes + a];
+          }
+          __syncwarp(ln.gm);
+        }
+      } else {
+        // ---------------------------------------------- one step on all lanes
+        last = step;
+        const PeRand<T, MIX> rd = rnd[step & (L - 1)];
+        // ---- Gibbs part 1: MH on t0 (Sec. 2.4), uniform prior on its grid range
+        T la0 = (T)NAN;
+        const T lu0 = rd.lu0;
+        if (M.sample_t0) {
+          const int Dm = fp32 ? __float2int_rn((float)(rd.z1 * inv_gT)) : __double2int_rn((double)(rd.z1 * inv_gT));
+          const int k0p = k0 + Dm;
+          if (Dm == 0) {
+            la0 = (T)0;
+          } else if (k0p < k0_lo || k0p > k0_hi) {
+            la0 = (T)-INFINITY;
           } else {
-            la = dnu + la_prior;
+            T part = (T)0;
+#pragma unroll 1
+            for (int k = ln.sl; k < N; k += L) {
+              const int j = W.list()[k];
+              part += pe_logphi<T>(M, j - k0p) - pe_logphi<T>(M, j - k0);
+            }
+            la0 = wsum(part, ln);
+          }
+          t0_acc = lu0 < la0;
+          if (t0_acc) k0 = k0p;
+        }
+        // ---- Gibbs part 2: one RJMCMC jump (Sec. 2.4)
+        jump = (N == 0) ? 0 : (rd.u3 < Jt ? 0 : (rd.u3 < (T)2 * Jt ? 1 : 2));
+        int st = 0, valid = 0, noop = 0, kk = -1, jp = -1, jm = -1;
+        if constexpr (MIX) e_m = rd.ep;
+        T la_prior = (T)0, la_fixed = (T)-INFINITY;
+        const T lu = rd.lu;
+        const T lphi_t0 = W.lPhi()[k0 - k0_lo];
+        if (jump == 0) {
+          if (N >= n_cap) {
+            st |= FSMP_ST_CAPACITY;
+          } else if (lphi_t0 > (T)-INFINITY) {
+            const T base = pe_cphi<T>(M, T_lo - 1 - k0), tot = pe_cphi<T>(M, T_hi - 1 - k0) - base;
+            jp = pe_birth_search<T, L>(M, T_lo, T_hi, k0, base, rd.u4 * tot, ln);
+            valid = jp >= T_lo;
+            la_prior = log_lambda0 + lphi_t0 - lgN[N + 1] + (N == 0 ? logJ : (T)0);
+          }
+        } else {
+          kk = fp32 ? __float2int_rd((float)(rd.u4 * (T)N)) : __double2int_rd((double)(rd.u4 * (T)N));
+          if (kk >= N) kk = N - 1;
+          jm = W.list()[kk];
+          if constexpr (MIX) e_m = W.le()[kk];
+          if (jump == 1) {
+            valid = 1;
+            la_prior = -log_lambda0 - lphi_t0 + lgN[N] - (N == 1 ? logJ : (T)0);
+          } else {
+            const int Dm = fp32 ? __float2int_rn((float)(rd.z2 * inv_gT)) : __double2int_rn((double)(rd.z2 * inv_gT));
+            const int jpl = jm + Dm;
+            bool same = Dm == 0;
+            if constexpr (MIX) same = same && rd.ep == e_m;
+            if (same) {  // same time and component: an accepted no-op
+              noop = 1;
+              la_fixed = (T)0;
+            } else if (jpl < T_lo || jpl >= T_hi || pe_logphi<T>(M, jpl - k0) == (T)-INFINITY) {
+              la_fixed = (T)-INFINITY;
+            } else {
+              jp = jpl;
+              valid = 1;
+              la_prior = pe_logphi<T>(M, jp - k0) - pe_logphi<T>(M, jm - k0);
+            }
           }
         }
+        // ---- scoring: the 2x2 quantities in PE space, then the 2x2 algebra in T
+        mv.jump = jump; mv.kk = kk; mv.jp = jp; mv.jm = jm; mv.np = 0;
+        // components of a_- and a_+; the absent one of a birth or death takes the other's values
+        // (its terms vanish)
+        mv.em = e_m;
+        mv.ep = 0;
+        if constexpr (MIX) mv.ep = jump == 1 ? e_m : rd.ep;
+        mv.aa = mv.vk = mv.ay = czero<C>();
+        mv.sp = Sup{0, 0, 0, 0};
+        T mmm = 0, mmp = 0, mpp = 0, gm = 0, gp = 0, em = 1;
+        if (valid) {
+          if (jump != 1) {
+            const Sup sp = pe_sup(M, n, jp);
+            mv.sp = sp;
+            mv.aa = xcorr<C>(M, tc, sp, 0);  // issued first: its table load overlaps the scan's
+            // PEs overlapping a_+, with b_q = a_q^T a_+
+            int np = 0;
+#pragma unroll 1
+            for (int base = 0; base < N; base += L) {
+              const int qi = base + ln.sl;
+              C bq = czero<C>();
+              if (qi < N) {
+                const int o = jp - W.list()[qi];
+                if (o > -M.Lt && o < M.Lt) bq = xcorr<C>(M, tc, sp, o);
+              }
+              const bool ov = cnz(bq);
+              const unsigned b = gballot(ov, ln);
+              if (ov) {
+                const int pos = np + __popc(b & ((1u << ln.sl) - 1u));
+                W.ovi()[pos] = qi;
+                W.ovb()[pos] = bq;
+              }
+              np += __popc(b);
+            }
+            __syncwarp(ln.gm);
+            mv.np = np;
+            // b^T C^-1 b over the lower triangle of the overlap block (lanes over its entries, the
+            // off-diagonal ones counted twice), b^T v, (C^-1 b)_k of an update and a_+^T y, then one
+            // reduction of the four over the group
+            T ayp = (T)0;
+#pragma unroll 1
+            for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) ayp += Vs[sp.ph + i * R] * W.y()[sp.w0 + i];
+            C qp = czero<C>(), ck = czero<C>();
+            T bvp = (T)0;
+            const int nt = tri(np);
+            TriWalk<L> tw;
+            int e = ln.sl;
+            // the products of two entries e, e + L at a time (BIG, C^-1 in the global slot: two
+            // such pairs, their loads ahead of their sums), added in order
+            constexpr int PE = BIG ? 4 : 2;
+#pragma unroll 1
+            for (; e < nt; e += PE * L) {
+              C cq[PE], ba[PE], bb[PE];
+              bool dg[PE];
+#pragma unroll
+              for (int u = 0; u < PE; ++u) {
+                const bool in = e + u * L < nt;  // beyond the triangle: zero terms
+                if (in) tw.at(tij, e + u * L);
+                const C c = Cp[tri(W.ovi()[tw.i]) + W.ovi()[tw.j]];
+                cq[u] = in ? c : czero<C>();
+                ba[u] = W.ovb()[tw.i];
+                bb[u] = W.ovb()[tw.j];
+                dg[u] = tw.i == tw.j;
+              }
+#pragma unroll
+              for (int u = 0; u < PE; u += 2) {
+                const Pk<C> t = pk_mul(pk2(cq[u], cq[u + 1]), pk_mul(pk2(ba[u], ba[u + 1]), pk2(bb[u], bb[u + 1])));
+                const C t0 = pk_first(t), t1 = pk_second(t);
+                qp = cadd(qp, dg[u] ? t0 : ctwice(t0));
+                qp = cadd(qp, dg[u + 1] ? t1 : ctwice(t1));
+              }
+            }
+#pragma unroll 1
+            for (int a = ln.sl; a < np; a += L) {
+              const C ba = W.ovb()[a];
+              bvp += (T)cnum(ba) * (T)cnum(W.v()[W.ovi()[a]]);
+              if (opaque(jump == 2)) ck = cfma(Cp[pk(kk, W.ovi()[a])], ba, ck);
+            }
+            gsum4<L, L>(qp, ck, bvp, ayp, ln);
+            const T bvT = bvp;  // b^T v at the scoring precision (the accept recomputes it)
+            const T ayT = ayp;
+            mv.ay = cfromf(ayT);
+            mpp = (T)cnum(csub(mv.aa, qp)) * ise2T;
+            gp = (ayT - bvT) * ise2T;
+            mmp = (T)cnum(ck);  // times 1 / sigma_-^2 below (update only)
+            words += (unsigned)(N + 2 * np + 2 * (sp.ihi - sp.ilo) + np * np + np);
+          }
+          if (jump != 0) {
+            const T iqm = CmT<T>::iq(M, mv.em);
+            mv.vk = W.v()[kk];
+            em = CmT<T>::r(M, mv.em) * (T)cnum(Cp[tri(kk) + kk]);
+            mmm = ((T)1 - em) * iqm;
+            gm = (T)cnum(mv.vk) * iqm;
+            mmp *= iqm;
+            words += 2;
+          }
+        }
+        T la = la_fixed;
+        if (valid) {
+          const PeScore<T> sc = pe_score<T, MIX>(M, mv.em, mv.ep, em, mmm, mmp, mpp, gm, gp);
+          dT = sc.dT;
+          dnu = sc.dnu;
+          st |= sc.st;
+          la = sc.ok ? dnu + la_prior : (T)-INFINITY;
+        }
+        const bool acc = lu < la;
+        apply = acc && valid && isfinite(la);
+        if (ln.sl == 0) {
+          if (st) S.status |= st;
+          if (trace)
+            pe_trace_record(trace + step, (double)la0, (double)lu0, (double)la, (double)lu, (double)dnu,
+                            N + (apply ? (jump == 0 ? 1 : (jump == 1 ? -1 : 0)) : 0), k0, jump,
+                            (M.sample_t0 ? 1 : 0) | (t0_acc ? 2 : 0) | (acc ? 4 : 0) | ((acc && noop) ? 8 : 0));
+        }
       }
-      const int acc = lu < la;
-      const int apply = acc && valid && isfinite(la);
 
       // ---- accepted move: C^-1, v, y and the PE list
       if (apply) {
         {
-          const AcceptOut<C> ao = pe_accept<T, BIG, L, MIX>(M, W, Vs, Cp, cap, Cg, mv, n, N, ln);
+          const AcceptOut<C> ao = pe_accept<T, BIG, L, MIX>(M, W, Cp, cap, Cg, mv, n, N, ln);
           Cp = ao.Cp;
           cap = ao.cap;
           N = ao.N;
-          words += ao.words;
+          words += (unsigned)ao.words;
         }
+        close_hold(S, last, burn_in, true, dT, dnu, ln.sl);
         C qs = czero<C>();
-        double ms = 0.0;  // sum of the PEs' means (the mixture; N mu_q for the dynode model)
+        double ms = M.cm_mu[0];  // the PEs' mean charge (the mixture: the sum of them)
+        if constexpr (MIX) ms = 0.0;
+#pragma unroll 1
         for (int i = ln.sl; i < N; i += L) {
-          qs = cadd(qs, W.v[i]);
-          if (mix) ms += M.cm_mu[W.le[i]];
+          qs = cadd(qs, W.v()[i]);
+          if constexpr (MIX) ms += M.cm_mu[W.le()[i]];
         }
-        qs = csum(qs, ln);
-        ms = mix ? wsum(ms, ln) : N * M.cm_mu[0];
+        qs = csum_m(qs, N, ln);
+        if constexpr (MIX) ms = wsum(ms, ln);
         if (ln.sl == 0) {
-          close_hold(S, step, burn_in);
-          S.q_cur = ms + c64(qs);
-          S.q_from = step;
+          S.q_from = last;
           // the PE removed (death, update) and the one added (birth, update)
           if (jump != 1) { S.St += abs(mv.jp); S.Se += mv.ep; }
           if (jump != 0) { S.St -= abs(mv.jm); S.Se -= mv.em; }
-          set_wasserstein(S, M.g, N, inv1);
-          S.logdet += (double)dT;
-          S.logL += (double)dnu;
           S.n_acc_refresh++;
         }
+        __syncwarp(ln.gm);
+        set_summaries<MIX>(S, M.g, N, ms, c64(qs), inv1, ln.sl);
         __syncwarp(ln.gm);
         if (fp32 && M.refresh_every > 0 && S.n_acc_refresh >= M.refresh_every) {
           const RefreshOut ro = pe_refresh<T, BIG, L, MIX>(M, W, Cp, ws, n_cap, w, S.wsq, n, N, ln);
           C qr = czero<C>();
-          for (int i = ln.sl; i < N; i += L) qr = cadd(qr, W.v[i]);
+#pragma unroll 1
+          for (int i = ln.sl; i < N; i += L) qr = cadd(qr, W.v()[i]);
           qr = csum(qr, ln);
           if (ln.sl == 0) {
             S.n_acc_refresh = 0;
             if (ro.ok) {
-              S.logdet = ro.logdet; S.logL = ro.logL;
+              S.sum[PeStats::kLogdet] = ro.logdet; S.sum[PeStats::kLogL] = ro.logL;
               S.drift_max = fmax(S.drift_max, ro.drift);
               if (ro.drift > M.drift_tol) S.status |= FSMP_ST_DRIFT;
               S.n_refresh++;
-              S.q_cur = ms + c64(qr);
+              S.cur[0] = fma(MIX ? 1.0 : (double)N, ms, c64(qr));
             } else {
               S.status |= FSMP_ST_DRIFT;
               S.refresh_fail++;
@@ -1648,22 +2254,16 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
         }
       }
 
-      // ---- bookkeeping of the decided step (the group's first lane)
-      if (ln.sl == 0) {
-        S.prop[jump]++;
-        if (t0f & 1) { S.prop_t0++; if (t0f & 2) S.acc_t0++; }
-        if (apply) S.acc[jump]++;
-        S.status |= st_a | st_c;
-        S.alg_words += words;
-        if (step >= burn_in) {
-          const long long Nn = N, kq = k0;
-          S.sN += Nn; S.sN2 += Nn * Nn; S.sK += kq; S.sK2 += kq * kq;
-          atomicAdd(hist + N, 1);  // no value returned: the lane does not wait on it
+      // ---- bookkeeping of the accepted step (of a batch) or of the step made alone
+      if (one) {
+        if (ln.sl < kCounts)
+          W.cnt()[ln.sl] += count_of(ln.sl, N, k0, last >= burn_in, words, jump, apply, t0_acc);
+        if (last >= burn_in) {
+          if (ln.sl == 0) atomicAdd(hist + N, 1);  // no value returned: the lane does not wait on it
+          if (peh) pe_hist_add(W, peh, N, T_lo, B.pe_hist_width, 1u, ln);
         }
-        if (trace) pe_trace_record(trace + step, (double)la0, (double)lu0, (double)la, (double)lu, (double)dnu, N, k0, jump,
-                                   t0f | (acc ? 4 : 0) | ((acc && noop) ? 8 : 0));
       }
-      if (peh && step >= burn_in) pe_hist_add<L>(peh, W.list, N, T_lo, B.pe_hist_width, ln);
+      step = last + 1;
       __syncwarp(ln.gm);
     }
 
@@ -1673,7 +2273,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
       const RefreshOut ro = pe_refresh<T, BIG, L, MIX>(M, W, Cp, ws, n_cap, w, S.wsq, n, N, ln);
       if (ln.sl == 0) {
         if (ro.ok) {
-          S.logdet = ro.logdet; S.logL = ro.logL;
+          S.sum[PeStats::kLogdet] = ro.logdet; S.sum[PeStats::kLogL] = ro.logL;
           S.drift_max = fmax(S.drift_max, ro.drift);
           if (ro.drift > M.drift_tol) S.status |= FSMP_ST_DRIFT;
           S.n_refresh++;
@@ -1682,24 +2282,35 @@ __global__ void __launch_bounds__(kPeMaxThreads, 4)
         }
       }
     }
+    if (ln.sl < kCounts) {  // the subgroups' counts together
+      unsigned long long t = W.cnt()[ln.sl];
+#pragma unroll 1
+      for (int i = 1; i < kSpec; ++i) t += W.cnt()[i * kCounts + ln.sl];
+      W.cnt()[ln.sl] = t;
+    }
+    __syncwarp(ln.gm);
+    close_hold(S, n_steps, burn_in, false, (T)0, (T)0, ln.sl);
+    __syncwarp(ln.gm);
     const double lam_hat = pe_lambda_mle<L>(hist, n_cap, lambda0, ln.sl, ln.gm);
     if (ln.sl == 0) {
-      close_hold(S, n_steps, burn_in);
       fsmp_summary o;
       o.lambda_hat = lam_hat;
       int ns = n_steps - burn_in;
       if (ns < 0) ns = 0;
       const double inv = ns > 0 ? 1.0 / ns : NAN;
-      const double mN = (double)S.sN * inv, mK = (double)S.sK * inv;
-      o.mean_N = mN; o.var_N = (double)S.sN2 * inv - mN * mN;
-      o.mean_t0 = t_origin + M.g * mK; o.var_t0 = M.g * M.g * ((double)S.sK2 * inv - mK * mK);
-      o.mean_Q = S.sQ * inv; o.var_Q = S.sQ2 * inv - o.mean_Q * o.mean_Q;
-      o.mean_wt = S.sWt * inv; o.var_wt = S.sWt2 * inv - o.mean_wt * o.mean_wt;
-      o.mean_we = S.sWe * inv; o.var_we = S.sWe2 * inv - o.mean_we * o.mean_we;
-      o.logL = S.logL; o.logdet = S.logdet;
-      o.drift_max = S.drift_max; o.alg_bytes = (double)S.alg_words * 8.0;
-      for (int k = 0; k < 3; ++k) { o.acc[k] = S.acc[k]; o.prop[k] = S.prop[k]; }
-      o.acc_t0 = S.acc_t0; o.prop_t0 = S.prop_t0; o.N_final = N; o.k0_final = k0;
+      const long long* const cnt = reinterpret_cast<const long long*>(W.cnt());
+      const double mN = (double)cnt[0] * inv, mK = (double)cnt[2] * inv;
+      o.mean_N = mN; o.var_N = (double)cnt[1] * inv - mN * mN;
+      o.mean_t0 = t_origin + M.g * mK; o.var_t0 = M.g * M.g * ((double)cnt[3] * inv - mK * mK);
+      o.mean_Q = S.sum[0] * inv; o.var_Q = S.sum[1] * inv - o.mean_Q * o.mean_Q;
+      o.mean_wt = S.sum[2] * inv; o.var_wt = S.sum[3] * inv - o.mean_wt * o.mean_wt;
+      o.mean_we = S.sum[4] * inv; o.var_we = S.sum[5] * inv - o.mean_we * o.mean_we;
+      o.logL = S.sum[PeStats::kLogL]; o.logdet = S.sum[PeStats::kLogdet];
+      o.drift_max = S.drift_max; o.alg_bytes = (double)W.cnt()[4] * 8.0;
+      o.prop[0] = (int)(unsigned)W.cnt()[5]; o.prop[1] = (int)(W.cnt()[5] >> 32);
+      o.prop[2] = n_steps - o.prop[0] - o.prop[1];
+      o.acc[0] = (int)(unsigned)W.cnt()[6]; o.acc[1] = (int)(W.cnt()[6] >> 32); o.acc[2] = (int)(unsigned)W.cnt()[7];
+      o.acc_t0 = (int)(W.cnt()[7] >> 32); o.prop_t0 = M.sample_t0 ? n_steps : 0; o.N_final = N; o.k0_final = k0;
       o.status = S.status; o.n_samples = ns; o.n_refresh = S.n_refresh; o.reserved = 0;
       *out = o;
       note_chain_done(B, wi);

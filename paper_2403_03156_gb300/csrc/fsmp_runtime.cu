@@ -123,6 +123,7 @@ struct fsmp_ctx {
   std::vector<PeSet> pe_sets;
   int pe_slots = 0, pe_warps = 4, pe_tile = 0, pe_lanes = 32;
   bool pe_lanes_free = false;  // pe_lanes left to fsmp_autotune
+  bool pe_tile_free = false;   // pe_tile neither given nor tuned
   size_t pe_c_stride = 0, pe_ws_stride = 0, pe_bytes = 0;
   std::atomic<long long> n_launches{0};  // chain-kernel launches
   std::mutex tune_mu;                    // serialises fsmp_autotune calls
@@ -252,30 +253,45 @@ void CUDART_CB pack_done_cb(void* arg) {
 
 // ---- device batch from arrays already on the device
 // Launch shape of the PE-space kernel for windows up to n_alloc: warps per CTA, lanes per chain,
-// the shared tile of C^-1, and resident CTAs per SM from the hardware's occupancy rule.
-int pe_chains_per_cta(const fsmp_ctx* c) { return c->pe_warps * (32 / c->pe_lanes); }
-int pe_shape(fsmp_ctx* c, int n_alloc, int* ctas, size_t* smem) {
-  *smem = pe_smem_bytes(c->M, n_alloc, c->pe_warps, c->pe_lanes, c->pe_tile);
-  if (*smem > (size_t)c->prop.sharedMemPerBlockOptin) return FSMP_ERR_INVALID;
-  int per_sm = pe_kernel_occupancy(c->p.precision, c->pe_warps * 32, *smem, pe_big(c->p.n_cap), c->pe_lanes,
+// the shared tile of C^-1, and resident CTAs per SM from the hardware's occupancy rule. Where the
+// context's tile and warps do not fit shared memory (but are within its limits), a smaller tile (down to 16 PEs) and then fewer
+// warps are taken, and in the end a smaller tile still: the results do not depend on either.
+struct PeShape {
+  int warps, tile, ctas;
+  size_t smem;
+};
+int pe_shape(const fsmp_ctx* c, int n_alloc, PeShape* s) {
+  const int tile = c->pe_tile_free ? std::min(c->p.n_cap, 32) : c->pe_tile;
+  if (pe_limit_bytes(c->M, n_alloc, c->pe_warps, c->pe_lanes, tile) > (size_t)c->prop.sharedMemPerBlockOptin)
+    return FSMP_ERR_INVALID;
+  s->warps = c->pe_warps;
+  s->tile = c->pe_tile;
+  for (;;) {
+    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, s->tile);
+    if (s->smem <= (size_t)c->prop.sharedMemPerBlockOptin) break;
+    const bool slots = c->pe_c_stride > 0;  // room for C^-1 beyond the tile
+    if (slots && s->tile > 16) s->tile = std::max(16, s->tile - 8);
+    else if (s->warps > 1) s->warps /= 2;
+    else if (slots && s->tile > 0) s->tile = std::max(0, s->tile - 8);
+    else return FSMP_ERR_INVALID;
+  }
+  int per_sm = pe_kernel_occupancy(c->p.precision, s->warps * 32, s->smem, pe_big(c->p.n_cap), c->pe_lanes,
                                    c->M.n_comp > 1);
   if (per_sm < 1) return FSMP_ERR_INVALID;
   if (c->p.pe_ctas_per_sm > 0) per_sm = std::min(per_sm, c->p.pe_ctas_per_sm);
-  *ctas = per_sm * c->prop.multiProcessorCount;
+  s->ctas = per_sm * c->prop.multiProcessorCount;
   return FSMP_OK;
 }
 
 int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   if (c->pe_sets.empty()) FAIL(FSMP_ERR_INVALID, "the PE-space kernel was not set up at fsmp_create");
   if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
-  int ctas = 0;
-  size_t smem = 0;
-  if (pe_shape(c, B.n_max, &ctas, &smem) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
-  const int cpc = pe_chains_per_cta(c);
-  ctas = std::min(ctas, c->pe_slots / cpc);
-  ctas = std::min(ctas, (B.n_waveforms + cpc - 1) / cpc);
+  PeShape s;
+  if (pe_shape(c, B.n_max, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
+  const int cpc = s.warps * (32 / c->pe_lanes);
+  const int ctas = std::min(std::min(s.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
   const fsmp_ctx::PeSet& ps = c->pe_sets[set];
-  cudaError_t e = launch_pe(c->M, B, c->pe_warps, c->pe_lanes, ctas, c->pe_tile, smem, ps.cinv, c->pe_c_stride,
+  cudaError_t e = launch_pe(c->M, B, s.warps, c->pe_lanes, ctas, s.tile, s.smem, ps.cinv, c->pe_c_stride,
                             ps.ws, c->pe_ws_stride, ps.hist, ps.counter, st);
   c->n_launches++;
   if (e != cudaSuccess) { set_error("launch_pe", cudaGetErrorString(e), __LINE__); return FSMP_ERR_CUDA; }
@@ -901,9 +917,13 @@ int fsmp_create(const fsmp_params* params, fsmp_ctx** out) {
   if (p.kernel == FSMP_KERNEL_PE) {
     c->pe_warps = p.threads_per_chain > 0 ? std::min(4, p.threads_per_chain / 32) : 4;
     const size_t esz = pe_c_entry_bytes(p.precision);
-    c->pe_tile = p.pe_tile > 0 ? std::min(p.pe_tile, p.n_cap) : std::min(p.n_cap, 32);
+    // default tile: 40 PEs leaves the L1 the global slots are read through its size (pile-up, 600
+    // chains: 85.6 ms, 89.4 with 48 and 94.7 with 32; the same for the serving model, n_cap 192)
+    c->pe_tile = p.pe_tile > 0 ? std::min(p.pe_tile, p.n_cap) : std::min(p.n_cap, 40);
     c->pe_lanes = p.pe_lanes > 0 ? p.pe_lanes : 32;
     c->pe_lanes_free = p.pe_lanes == 0 && pe_lanes_ok(16, p.n_cap);
+    c->pe_tile_free = p.pe_tile == 0;
+    c->pe_c_stride = c->pe_tile < p.n_cap ? pe_c_entries(p.n_cap) : 0;
     CK(pe_kernel_attributes(p.precision, max_smem));
     int slots = 0;
     const int lanes0 = c->pe_lanes;
@@ -911,15 +931,13 @@ int fsmp_create(const fsmp_params* params, fsmp_ctx** out) {
       if (lanes != lanes0 && !c->pe_lanes_free) continue;
       c->pe_lanes = lanes;
       for (int nn : {std::min(64, p.n_max), p.n_max}) {
-        int ctas = 0;
-        size_t sm = 0;
-        if (pe_shape(c.get(), nn, &ctas, &sm) == FSMP_OK) slots = std::max(slots, ctas * pe_chains_per_cta(c.get()));
+        PeShape s;
+        if (pe_shape(c.get(), nn, &s) == FSMP_OK) slots = std::max(slots, s.ctas * s.warps * (32 / lanes));
       }
     }
     c->pe_lanes = lanes0;
     if (slots < 1) FAIL(FSMP_ERR_INVALID, "n_max too large for the PE-space kernel");
     c->pe_slots = slots;
-    c->pe_c_stride = c->pe_tile < p.n_cap ? pe_c_entries(p.n_cap) : 0;
     // the FP64 rebuild runs in FP32 mode every K accepts, and in both modes for a chain that
     // starts from a given z
     c->pe_ws_stride = pe_ws_slot_doubles(p.n_cap);
@@ -1095,11 +1113,12 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   CK(cudaEventCreate(&e1));
   const int set = (int)c->streams.size();
   const int tile0 = c->pe_tile, warps0 = c->pe_warps, ctas0 = c->p.pe_ctas_per_sm, lanes0 = c->pe_lanes;
+  const bool tfree0 = c->pe_tile_free;
+  c->pe_tile_free = false;  // the trials run in the shapes they name, later launches in the chosen one
   auto trial = [&](int lanes, int tile, int warps, int ctas, double* rate) -> int {
     c->pe_lanes = lanes; c->pe_tile = tile; c->pe_warps = warps; c->p.pe_ctas_per_sm = ctas;
-    int cc = 0;
-    size_t sm = 0;
-    if (pe_shape(c, B.n_max, &cc, &sm) != FSMP_OK) { *rate = -1.0; return FSMP_OK; }
+    PeShape s;
+    if (pe_shape(c, B.n_max, &s) != FSMP_OK || s.warps != warps || s.tile != tile) { *rate = -1.0; return FSMP_OK; }
     float best_ms = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {  // the first run warms the caches and the code
       if (cudaEventRecord(e0, st) != cudaSuccess) return FSMP_ERR_CUDA;
@@ -1161,6 +1180,7 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   cudaFree(scratch);
   if (rc != FSMP_OK) {
     c->pe_lanes = lanes0; c->pe_tile = tile0; c->pe_warps = warps0; c->p.pe_ctas_per_sm = ctas0;
+    c->pe_tile_free = tfree0;
     return rc;
   }
   c->pe_lanes = bl; c->pe_tile = bt; c->pe_warps = bw; c->p.pe_ctas_per_sm = bc;
@@ -1200,11 +1220,10 @@ int fsmp_get_info(fsmp_ctx* c, fsmp_info* o) {
   o->L_V = c->M.L_V;
   o->n_smem_max = c->n_smem_max;
   if (c->p.kernel == FSMP_KERNEL_PE) {  // pe_lanes lanes per chain, pe_warps warps per CTA
-    int ctas = 0;
-    size_t sm = 0;
-    if (pe_shape(c, c->p.n_max, &ctas, &sm) == FSMP_OK) {
+    PeShape s;
+    if (pe_shape(c, c->p.n_max, &s) == FSMP_OK) {
       o->threads_per_chain = c->pe_lanes;
-      o->ctas_per_sm = ctas / c->prop.multiProcessorCount;
+      o->ctas_per_sm = s.ctas / c->prop.multiProcessorCount;
     }
   } else {
     LaunchShape s;
