@@ -306,10 +306,10 @@ cudaError_t launch_pe(const DevModel& M, const BatchView& B, int warps, int lane
 // device function the chain kernels end with (testing aid; fsmp_pe.cu).
 cudaError_t launch_lambda_mle(const int* h, int n_hist, int n_max, const double* lambda0, double* out, int lanes,
                               cudaStream_t st);
-// LucyDDM (fsmp_lucy.cu): shared memory per CTA for windows up to n_alloc; the kernel taps
+// LucyDDM (fsmp_lucy.cu): the shared memory that limits n_alloc; the kernel taps
 // v(m) = V(m dt) / S, padded to whole groups of four, and S (on the device); the deconvolution
 // launch, given the taps in host memory (they travel in the kernel's parameters).
-size_t lucy_smem_bytes(int LV, int n_alloc);
+size_t lucy_limit_bytes(int LV, int n_alloc);
 cudaError_t lucy_kernel_attributes(int max_smem);
 cudaError_t launch_lucy_taps(const float* V32, int LV, int R, float* v4, float* S_dev, cudaStream_t st);
 cudaError_t launch_lucy(const float* v4_host, float S, int LV, int R, double dt, double g, int n_waveforms, int n_alloc,

@@ -1073,7 +1073,7 @@ int fsmp_lucyddm(fsmp_ctx* c, const fsmp_lucy_batch* b, void* stream) {
     FAIL(FSMP_ERR_INVALID, "fsmp_lucyddm: bad arguments");
   const int n_alloc = b->n_max_hint > 0 ? b->n_max_hint : c->p.n_max;
   if (n_alloc > c->p.n_max) FAIL(FSMP_ERR_INVALID, "fsmp_lucyddm: window longer than n_max");
-  if (lucy_smem_bytes(c->M.L_V, n_alloc) > (size_t)c->prop.sharedMemPerBlockOptin)
+  if (lucy_limit_bytes(c->M.L_V, n_alloc) > (size_t)c->prop.sharedMemPerBlockOptin)
     FAIL(FSMP_ERR_INVALID, "fsmp_lucyddm: window too long for shared memory");
   { cudaError_t e_ = cudaSetDevice(c->p.device); if (e_ != cudaSuccess) { set_error("cudaSetDevice", cudaGetErrorString(e_), __LINE__); return FSMP_ERR_CUDA; } }
   cudaError_t e = launch_lucy(c->lucy_v4_host.data(), c->lucy_S, c->M.L_V, c->M.R, c->M.dt, c->M.g, b->n_waveforms, n_alloc,
