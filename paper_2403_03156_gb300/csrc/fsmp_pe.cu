@@ -6,14 +6,15 @@
 
 namespace fsmp {
 
-size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns) {
-  const int chains = warps * (32 / lanes);
+size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns, bool team) {
+  const int chains = team ? 1 : warps * (32 / lanes);
+  const size_t cmd = team ? kTeamBytes : 0;
   auto bytes = [&](auto big, auto lane_count, auto mix) {
     constexpr bool BIG = decltype(big)::value, MIX = decltype(mix)::value;
     constexpr int L = decltype(lane_count)::value;
     if (M.precision == FSMP_FP64)
       return pe_block_bytes<double>(M) + chains * pe_chain_bytes<double, BIG, L, MIX>(M.n_cap, n_alloc, M.win_extra, Ns);
-    return pe_block_bytes<float>(M) + chains * pe_chain_bytes<float, BIG, L, MIX>(M.n_cap, n_alloc, M.win_extra, Ns);
+    return pe_block_bytes<float>(M) + cmd + chains * pe_chain_bytes<float, BIG, L, MIX>(M.n_cap, n_alloc, M.win_extra, Ns);
   };
   using std::false_type;
   using std::true_type;
@@ -59,15 +60,17 @@ bool pe_big(int n_cap) { return n_cap > 192; }
 // Lanes per chain the kernel is built for: 32, and 16 where chains are small (not BIG).
 bool pe_lanes_ok(int lanes, int n_cap) { return lanes == 32 || (lanes == 16 && !pe_big(n_cap)); }
 
+bool pe_team_ok(int precision, int lanes) { return precision != FSMP_FP64 && lanes == 32; }
+
 
 cudaError_t pe_kernel_attributes(int precision, int max_smem) {
   const cudaError_t e = pe_set_attributes<false>(precision, max_smem);
   return e != cudaSuccess ? e : pe_mix_attributes(precision, max_smem);
 }
 
-int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool mix) {
-  if (mix) return pe_mix_occupancy(precision, threads, smem, lanes);
-  return pe_occupancy<false>(precision, threads, smem, big, lanes);
+int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool mix, bool team) {
+  if (mix) return pe_mix_occupancy(precision, threads, smem, lanes, team);
+  return pe_occupancy<false>(precision, threads, smem, big, lanes, team);
 }
 
 // lambda_FSMP of given N histograms (testing aid): the device function every chain ends with,
@@ -94,12 +97,14 @@ cudaError_t launch_lambda_mle(const int* h, int n_hist, int n_max, const double*
 
 cudaError_t launch_pe(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                       void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                      cudaStream_t st) {
+                      bool team, cudaStream_t st) {
   if (hist == nullptr || !pe_lanes_ok(lanes, M.n_cap)) return cudaErrorInvalidValue;
+  if (team && (!pe_team_ok(M.precision, lanes) || warps != kTeam)) return cudaErrorInvalidValue;
   if (M.n_comp > 1)
-    return pe_mix_launch(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter, st);
+    return pe_mix_launch(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter, team,
+                         st);
   return pe_launch<false>(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter,
-                          pe_big(M.n_cap), st);
+                          pe_big(M.n_cap), team, st);
 }
 
 }  // namespace fsmp

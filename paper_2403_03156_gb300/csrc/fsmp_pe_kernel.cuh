@@ -782,15 +782,200 @@ struct RefreshOut {
   double logdet, logL, drift;
 };
 
+// Teams. A chain of more than kSpecPes PEs spends nearly all of its step waiting for C^-1: one
+// warp keeps some hundred gathers in flight, and a launch of few chains ends when its longest one
+// does. With TW = kTeam the CTA is one chain: warp 0 runs it, and the other warps take part where a
+// step reads or writes all of C^-1 or rebuilds it. They wait at a barrier for the next command,
+// do their share, and meet again. Entries, rows and sums keep their operations and their order
+// (a sum of the scoring stays the sum of 32 partial sums), so the results are the same bit for bit.
+// 1000 pile-up chains x 2000 steps: 600 ms with a warp per chain, 255 with a team; a burst of 64
+// events of up to 100 PEs a channel: 104 and 51; 777 uneven windows x 1000 steps: 16.9 and 10.7.
+// Bound now: the latency of C^-1's gathers from L2 and of the sums' dependent additions, and the
+// FP64 pipe of the rebuilds. 4 CTAs per SM (128 registers): with 3, 3000 uneven windows take 18.8
+// ms against 16.4 and pile-up the same.
+constexpr int kTeam = 4;
+enum TeamOp { kOpExit, kOpScore, kOpRows, kOpUpdate, kOpRefresh };
+template <typename C> struct PeTeam {
+  C part[32];          // scoring: the partial sums of b^T C^-1 b
+  double red[kTeam][2];  // refresh: the warps' largest drift and entry
+  C* Cp;
+  double* ws;
+  const float* w;
+  double wsq;
+  C nig, idl;
+  int op, N, np, jump, kk, n, ok;
+};
+constexpr unsigned kTeamBytes = 640;
+// the command block: behind the block tables, before the chain
+template <typename T> __device__ __forceinline__ PeTeam<typename PeTab<T>::C>& pe_team(const DevModel& M) {
+  static_assert(sizeof(PeTeam<typename PeTab<T>::C>) <= kTeamBytes || sizeof(T) == 8, "the command block");
+  return *reinterpret_cast<PeTeam<typename PeTab<T>::C>*>(pe_smem + pe_block_bytes<T>(M));
+}
+__device__ __forceinline__ void team_bar() {
+  __syncwarp();
+  asm volatile("bar.sync 1, %0;" ::"n"(kTeam * 32) : "memory");
+}
+// the team's threads (TW = 1: the chain's lanes) meet
+template <int TW, int L> __device__ __forceinline__ void team_sync(const Lanes<L> ln) {
+  if constexpr (TW > 1) team_bar();
+  else __syncwarp(ln.gm);
+}
+// (i, j) of packed entries e, e + S, e + 2 S, ... (rows beyond the table are longer than 32)
+template <int S> struct TeamWalk {
+  int i = 0, j = 0;
+  __device__ __forceinline__ void at(const unsigned short* __restrict__ tij, int e) {
+    if (e < kTriTab) {
+      const int t = tij[e];
+      i = t >> 8;
+      j = t & 255;
+    } else {
+      j += S;
+      while (j > i) {
+        j -= i + 1;
+        ++i;
+      }
+    }
+  }
+};
+
+// b^T C^-1 b: partial sum l (of entries l, l + 32, ..) on four neighbouring threads, each of which
+// takes every fourth product; all four add them up in order.
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void team_score(const DevModel& M, const PeChain<T, BIG, L, MIX> W) {
+  using C = typename PeTab<T>::C;
+  PeTeam<C>& tm = pe_team<T>(M);
+  const unsigned short* const tij = pe_tij();
+  const C* const Cp = tm.Cp;
+  const int nt = tri(tm.np), lane = threadIdx.x & 31, r = lane & 3, l = (threadIdx.x >> 5) * 8 + (lane >> 2);
+  constexpr int U = 4;  // products of a thread per pass, their loads ahead of the sums
+  TeamWalk<128> tw;
+  C acc = czero<C>();
+#pragma unroll 1
+  for (int base = 0; base < nt; base += U * 128) {
+    C t[U];
+    int dg = 0;
+    {
+      C cq[U], ba[U], bb[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = base + u * 128 + r * 32 + l;
+        const bool in = e < nt;  // beyond the triangle: zero terms
+        if (in) tw.at(tij, e);
+        const C c = Cp[tri(W.ovi()[tw.i]) + W.ovi()[tw.j]];
+        cq[u] = in ? c : czero<C>();
+        ba[u] = W.ovb()[tw.i];
+        bb[u] = W.ovb()[tw.j];
+        dg |= (tw.i == tw.j) << u;
+      }
+#pragma unroll
+      for (int u = 0; u < U; u += 2) {
+        const Pk<C> p = pk_mul(pk2(cq[u], cq[u + 1]), pk_mul(pk2(ba[u], ba[u + 1]), pk2(bb[u], bb[u + 1])));
+        const C t0 = pk_first(p), t1 = pk_second(p);
+        t[u] = (dg >> u) & 1 ? t0 : ctwice(t0);
+        t[u + 1] = (dg >> (u + 1)) & 1 ? t1 : ctwice(t1);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc = cadd(acc, cshfl<4>(t[u], q, 0xffffffffu));
+  }
+  if (r == 0) tm.part[l] = acc;
+}
+
+// u' before the removed PE's term: row i of C^-1 times b~, a thread per row
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void team_rows(const DevModel& M, const PeChain<T, BIG, L, MIX> W) {
+  using C = typename PeTab<T>::C;
+  const PeTeam<C>& tm = pe_team<T>(M);
+  const C* const Cp = tm.Cp;
+  const int N = tm.N, np = tm.np;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < N; i += kTeam * 32) {
+    if constexpr (BIG) {
+      W.uv()[i] = dot_row4<C>(Cp, i, W.ovi(), W.ovb(), np);
+    } else {
+      C acc = czero<C>();
+      int a = 0;
+#pragma unroll 1
+      for (; a + 3 < np; a += 4) {
+        C x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = Cp[pk(i, W.ovi()[a + u])];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = cfma(x[u], W.ovb()[a + u], acc);
+      }
+#pragma unroll 1
+      for (; a < np; ++a) acc = cfma(Cp[pk(i, W.ovi()[a])], W.ovb()[a], acc);
+      W.uv()[i] = acc;
+    }
+  }
+}
+
+// The accepted move's pass over C^-1 (see pe_accept), entries over the team's threads. A pass
+// reads an entry only where it writes it, or in the last row for a death (which is not written).
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void team_update(const DevModel& M, const PeChain<T, BIG, L, MIX> W) {
+  using C = typename PeTab<T>::C;
+  const PeTeam<C>& tm = pe_team<T>(M);
+  const unsigned short* const tij = pe_tij();
+  C* const Cp = tm.Cp;
+  const int N = tm.N, jump = tm.jump, kk = tm.kk;
+  const bool has_m = jump != 0, has_p = jump != 1;
+  const int Nout = N + (jump == 0 ? 1 : (jump == 1 ? -1 : 0)), last = N - 1;
+  const int s = jump == 0 ? N : (jump == 2 ? kk : -1), kmap = jump == 1 ? kk : -1;
+  const int ne = tri(Nout);
+  const C nig = tm.nig, idl = tm.idl;
+  const C* const cv = W.cv();
+  const C* const cvn = BIG ? W.cv() : W.cvn();
+  const C* const uv = W.uv();
+  const C* const uvd = W.ovb();
+  constexpr int U = 4, S = kTeam * 32;
+  TeamWalk<S> tw;
+#pragma unroll 1
+  for (int e = threadIdx.x; e < ne; e += U * S) {
+    int ii[U], jj[U];
+    C x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (e + u * S < ne) tw.at(tij, e + u * S);
+      ii[u] = tw.i;
+      jj[u] = tw.j;
+      x[u] = Cp[pk(tw.i == kmap ? last : tw.i, tw.j == kmap ? last : tw.j)];
+    }
+#pragma unroll
+    for (int u = 0; u < U; u += 2) {
+      const int i = ii[u], j = jj[u], i2 = ii[u + 1], j2 = jj[u + 1];
+      Pk<C> y = pk2(x[u], x[u + 1]);
+      if (has_m) {
+        Pk<C> cj = pk2(cvn[j == kmap ? last : j], cvn[j2 == kmap ? last : j2]);
+        if constexpr (BIG) cj = pk_mul(cj, pk2(nig, nig));
+        y = pk_fma(pk2(cv[i == kmap ? last : i], cv[i2 == kmap ? last : i2]), cj, y);
+      }
+      if (has_p) y = pk_fma(pk2(uv[i], uv[i2]), pk2(uvd[j], uvd[j2]), y);
+      C y0 = pk_first(y), y1 = pk_second(y);
+      if (has_p) {
+        if (i == s || j == s) y0 = i == j ? idl : cneg(uvd[i == s ? j : i]);
+        if (i2 == s || j2 == s) y1 = i2 == j2 ? idl : cneg(uvd[i2 == s ? j2 : i2]);
+      }
+      if (e + u * S < ne) Cp[e + u * S] = y0;
+      if (e + (u + 1) * S < ne) Cp[e + (u + 1) * S] = y1;
+    }
+  }
+}
+
 // FP64 rebuild of C^-1, v, y, log|Sigma| and the log-likelihood from the PE list (FP32 mode).
 // ok = 0 (state untouched) if C is not numerically positive definite. Arguments are passed by
-// value (no address of the caller's locals escapes, so they stay in registers).
-template <typename T, bool BIG, int L, bool MIX>
-__device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T, BIG, L, MIX> W, typename PeTab<T>::C* Cp,
+// value (no address of the caller's locals escapes, so they stay in registers). TW > 1: every warp
+// of the team calls (see PeTeam); the outputs are warp 0's.
+template <typename T, bool BIG, int L, bool MIX, int TW>
+__device__ __noinline__ RefreshOut pe_refresh_part(const DevModel& M, const PeChain<T, BIG, L, MIX> W, typename PeTab<T>::C* Cp,
                                               double* ws, int n_cap, const float* w, double wsq, int n,
                                               int N, const Lanes<L> ln) {
   using C = typename PeTab<T>::C;
   RefreshOut out{0, 0.0, 0.0, 0.0};
+  const int wp = TW > 1 ? (int)(threadIdx.x >> 5) : 0, tl = wp * L + ln.sl;  // warp and thread of the team
+  constexpr int LT = L * TW;
   const int ws_ld = N > 0 ? N : 1;
   constexpr int SB = BIG ? kSweepBlock : kSweepBlock / 2;  // fewer registers in the compact variant
   const size_t lv = pe_ws_a2(n_cap);
@@ -810,7 +995,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
   // caller registers around the call, which the compact variant cannot spare.
   constexpr int RC = BIG ? 4 : 1, RG = BIG ? 4 : 1;
 #pragma unroll 1
-  for (int j = ln.sl; j < N; j += L) {
+  for (int j = tl; j < N; j += LT) {
     const int jj = W.list()[j];
 #pragma unroll 1
     for (int i0 = j; i0 < N; i0 += RC) {
@@ -829,13 +1014,13 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
       }
     }
   }
-  __syncwarp(ln.gm);
+  team_sync<TW>(ln);
   // With y = w - sum_k mu_k a_k: h = A^T y = A^T w - (A^T A) m (m the PEs' means), and
   // y^T y = w^T w - 2 m^T A^T w + m^T A^T A m -- no FP64 copy of y is needed. The dynode
   // model factors its single mean out.
   double awt = 0.0, rst = 0.0;
 #pragma unroll 1
-  for (int k = ln.sl; k < N; k += L) {
+  for (int k = tl; k < N; k += LT) {
     const Sup s = pe_sup(M, n, W.list()[k]);
     // the loops' loads go four at a time ahead of their (unchanged) sums
     double a0 = 0.0, a1 = 0.0;
@@ -880,8 +1065,13 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
 #pragma unroll 1
       for (; j < N; ++j) hs = fma(c_kj(j), M.cm_mu[W.le()[j]], hs);
       h[k] = aw - hs;
-      awt = fma(mk, aw, awt);
-      rst = fma(mk, hs, rst);
+      if constexpr (TW > 1) {
+        rowk[k] = aw;
+        P[k] = hs;
+      } else {
+        awt = fma(mk, aw, awt);
+        rst = fma(mk, hs, rst);
+      }
     } else {
       double rs = -r;
 #pragma unroll 1
@@ -894,18 +1084,40 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
       }
 #pragma unroll 1
       for (; j < N; ++j) rs += c_kj(j);
-      h[k] = aw - mu * rs;
-      awt += aw;
-      rst += rs;
+      h[k] = fma(-mu, rs, aw);
+      if constexpr (TW > 1) {
+        rowk[k] = aw;
+        P[k] = rs;
+      } else {
+        awt += aw;
+        rst += rs;
+      }
+    }
+  }
+  if constexpr (TW > 1) {  // the sums in the order in which one warp adds them
+    team_bar();
+#pragma unroll 1
+    for (int k = ln.sl; k < N; k += L) {
+      const double aw = rowk[k], rs = P[k];
+      if (mix) {
+        const double mk = M.cm_mu[W.le()[k]];
+        awt = fma(mk, aw, awt);
+        rst = fma(mk, rs, rst);
+      } else {
+        awt += aw;
+        rst += rs;
+      }
     }
   }
   awt = wsum(awt, ln);
   rst = wsum(rst, ln);
-  const double yy = mix ? wsq - 2.0 * awt + rst : wsq - 2.0 * mu * awt + mu * mu * rst;
+  // (roundings written out, so that every instance of this function gives the same bits)
+  const double yy = mix ? fma(-2.0, awt, wsq) + rst : fma(mu * mu, rst, fma(-2.0 * mu, awt, wsq));
   // the FP32 residual, each sample summed in FP64 over the PEs that cover it, in list order: PE
   // by PE with lanes over its support samples, into an FP64 copy of the window held in the
   // sweep's panel buffers (free until the sweep); sample by sample where the window does not fit
-  if (n <= 2 * kSweepBlock * (int)lv) {
+  // (and by a team, whose threads have few samples each)
+  if (TW == 1 && n <= 2 * kSweepBlock * (int)lv) {
     double* yd = P;  // P and Pn are contiguous
 #pragma unroll 1
     for (int x = ln.sl; x < n; x += L) yd[x] = (double)w[x];
@@ -922,7 +1134,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
     for (int x = ln.sl; x < n; x += L) W.y()[x] = (T)yd[x];
   } else {
 #pragma unroll 1
-    for (int x = ln.sl; x < n; x += L) {
+    for (int x = tl; x < n; x += LT) {
       double yv = (double)w[x];
 #pragma unroll 1
       for (int k = 0; k < N; ++k) {
@@ -932,7 +1144,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
       W.y()[x] = (T)yv;
     }
   }
-  __syncwarp(ln.gm);
+  team_sync<TW>(ln);
   // Inversion by the symmetric sweep operator (Gauss-Jordan with diagonal pivots, kept
   // symmetric): sweeping pivot p maps A_pp -> -1/A_pp, A_pj -> A_pj/A_pp, A_ip -> A_ip/A_pp and
   // A_ij -> A_ij - A_ip A_pj/A_pp. Sweeps commute, sweeping every index leaves -C^-1, and only
@@ -952,43 +1164,56 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
     // the diagonal block A_KK swept on its own, lane r holding its row r in full; each pivot's
     // row goes to the other lanes by shuffles
     const int rl = ln.sl;
-    double kr[SB];
-#pragma unroll
-    for (int c = 0; c < SB; ++c)
-      kr[c] = (rl < nb && c < nb)
-                  ? *(c <= rl ? A + (size_t)(k0 + rl) * ws_ld + k0 + c : A + (size_t)(k0 + c) * ws_ld + k0 + rl)
-                  : 0.0;
-#pragma unroll
-    for (int q = 0; q < SB; ++q) {
-      if (q < nb) {
-        const double piv = __shfl_sync(ln.gm, kr[q], q, L);
-        if (!(piv > 0.0) || !isfinite(piv)) return out;
-        const double ip = 1.0 / piv;
-        int ex;
-        pm *= frexp(piv, &ex);
-        pe += ex;
-        pm = frexp(pm, &ex);
-        pe += ex;
-        const double fr = kr[q] * ip;  // A_rp / pivot for this lane's row r
-        double aq[SB];
-#pragma unroll
-        for (int c = 0; c < SB; ++c) aq[c] = __shfl_sync(ln.gm, kr[c], q, L);
-#pragma unroll
-        for (int c = 0; c < SB; ++c)
-          kr[c] = (rl == q) ? (c == q ? -ip : aq[c] * ip) : (c == q ? fr : fma(-fr, aq[c], kr[c]));
-        if (rl < nb) F[q * SB + rl] = (rl == q) ? ip : fr;
-      }
-    }
-    if (rl < nb) {
+    if (TW == 1 || wp == 0) {
+      bool bad = false;
+      double kr[SB];
 #pragma unroll
       for (int c = 0; c < SB; ++c)
-        if (c <= rl) A[(size_t)(k0 + rl) * ws_ld + k0 + c] = kr[c];
+        kr[c] = (rl < nb && c < nb)
+                    ? *(c <= rl ? A + (size_t)(k0 + rl) * ws_ld + k0 + c : A + (size_t)(k0 + c) * ws_ld + k0 + rl)
+                    : 0.0;
+#pragma unroll
+      for (int q = 0; q < SB; ++q) {
+        if (q < nb) {
+          const double piv = __shfl_sync(ln.gm, kr[q], q, L);
+          if (!(piv > 0.0) || !isfinite(piv)) {
+            if constexpr (TW == 1) return out;
+            bad = true;
+            break;
+          }
+          const double ip = 1.0 / piv;
+          int ex;
+          pm *= frexp(piv, &ex);
+          pe += ex;
+          pm = frexp(pm, &ex);
+          pe += ex;
+          const double fr = kr[q] * ip;  // A_rp / pivot for this lane's row r
+          double aq[SB];
+#pragma unroll
+          for (int c = 0; c < SB; ++c) aq[c] = __shfl_sync(ln.gm, kr[c], q, L);
+#pragma unroll
+          for (int c = 0; c < SB; ++c)
+            kr[c] = (rl == q) ? (c == q ? -ip : aq[c] * ip) : (c == q ? fr : fma(-fr, aq[c], kr[c]));
+          if (rl < nb) F[q * SB + rl] = (rl == q) ? ip : fr;
+        }
+      }
+      if (rl < nb) {
+#pragma unroll
+        for (int c = 0; c < SB; ++c)
+          if (c <= rl) A[(size_t)(k0 + rl) * ws_ld + k0 + c] = kr[c];
+      }
+      if constexpr (TW > 1) {
+        if (ln.sl == 0) pe_team<T>(M).ok = !bad;
+      }
     }
-    __syncwarp(ln.gm);
+    team_sync<TW>(ln);
+    if constexpr (TW > 1) {
+      if (!pe_team<T>(M).ok) return out;
+    }
     // the panel A_Kj of every column j outside the block: P_j. keeps it as it was, then the
     // block's pivots are applied to it in registers and it goes to Pn_j. and back into A
 #pragma unroll 1
-    for (int j = ln.sl; j < N; j += L) {
+    for (int j = tl; j < N; j += LT) {
       if (j >= k0 && j < k1) continue;
       double b[SB];
 #pragma unroll
@@ -1011,7 +1236,7 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
         if (q < nb) *(j < k0 ? A + (size_t)(k0 + q) * ws_ld + j : A + (size_t)j * ws_ld + k0 + q) = b[q];
       }
     }
-    __syncwarp(ln.gm);
+    team_sync<TW>(ln);
     // every entry (i, j), i >= j, outside the block's rows and columns: lanes over a group of L
     // columns, the rows in step across the lanes (a row's loads coalesce and its P row is one
     // broadcast), RG rows at a time so that their loads overlap
@@ -1029,18 +1254,18 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
       double xn[RG];
 #pragma unroll
       for (int t = 0; t < RG; ++t) {
-        const int r = row(t);
-        xn[t] = (jv && t < nr && r >= j) ? A[(size_t)r * ws_ld + j] : 0.0;
+        const int t1 = wp * RG + t, r = row(t1);
+        xn[t] = (jv && t1 < nr && r >= j) ? A[(size_t)r * ws_ld + j] : 0.0;
       }
 #pragma unroll 1
-      for (int t0 = 0; t0 < nr; t0 += RG) {
+      for (int t0 = wp * RG; t0 < nr; t0 += TW * RG) {
         double x[RG];
         int rr[RG];
 #pragma unroll
         for (int t = 0; t < RG; ++t) {
           x[t] = xn[t];
           rr[t] = row(min(t0 + t, nr - 1));
-          const int tt = t0 + RG + t, r = row(tt);
+          const int tt = t0 + TW * RG + t, r = row(tt);
           xn[t] = (jv && tt < nr && r >= j) ? A[(size_t)r * ws_ld + j] : 0.0;
         }
 #pragma unroll
@@ -1058,13 +1283,13 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
           if (jv && t0 + t < nr && rr[t] >= j) A[(size_t)rr[t] * ws_ld + j] = x[t];
       }
     }
-    __syncwarp(ln.gm);
+    team_sync<TW>(ln);
   }
-  const double logdetC = log(pm) + (double)pe * 0.6931471805599453;
+  const double logdetC = fma((double)pe, 0.6931471805599453, log(pm));
   // v = C^-1 h = -A h (entry (i, j) of the symmetric A from the lower triangle; lanes over rows;
   // BIG: four partial sums)
 #pragma unroll 1
-  for (int i = ln.sl; i < N; i += L) {
+  for (int i = tl; i < N; i += LT) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     auto a_ij = [&](int j) { return *(j < i ? A + (size_t)i * ws_ld + j : A + (size_t)j * ws_ld + i); };
     int j = 0;
@@ -1079,21 +1304,21 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
     for (; j < N; ++j) s0 = fma(a_ij(j), h[j], s0);
     rowk[i] = -((s0 + s1) + (s2 + s3));
   }
-  __syncwarp(ln.gm);
+  team_sync<TW>(ln);
   double hv = 0.0;
 #pragma unroll 1
-  for (int i = ln.sl; i < N; i += L) hv += h[i] * rowk[i];
+  for (int i = ln.sl; i < N; i += L) hv = fma(h[i], rowk[i], hv);
   hv = wsum(hv, ln);
   // drift of the incremental state, then the refreshed state (packed lower triangle)
   double dmax = 0.0, amax = 0.0;
   constexpr int RD = BIG ? 4 : 1;  // entries per lane at a time, their loads ahead of their stores
   const int nt = tri(N);
 #pragma unroll 1
-  for (int e0 = ln.sl; e0 < nt; e0 += RD * L) {
+  for (int e0 = tl; e0 < nt; e0 += RD * LT) {
     double nv[RD], ov[RD];
 #pragma unroll
     for (int u = 0; u < RD; ++u) {
-      const int e = e0 + u * L;
+      const int e = e0 + u * LT;
       nv[u] = ov[u] = 0.0;
       if (e < nt) {
         int i, j;
@@ -1104,12 +1329,27 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
     }
 #pragma unroll
     for (int u = 0; u < RD; ++u) {
-      const int e = e0 + u * L;
+      const int e = e0 + u * LT;
       if (e < nt) {
         dmax = fmax(dmax, fabs(nv[u] - ov[u]));
         amax = fmax(amax, fabs(nv[u]));
         Cp[e] = cfrom64<C>(nv[u]);
       }
+    }
+  }
+  if constexpr (TW > 1) {  // the warps' largest drift and entry; what follows is warp 0's
+    PeTeam<C>& tm = pe_team<T>(M);
+    dmax = wmax(dmax, ln); amax = wmax(amax, ln);
+    if (ln.sl == 0) {
+      tm.red[wp][0] = dmax;
+      tm.red[wp][1] = amax;
+    }
+    team_bar();
+    if (wp > 0) return out;
+#pragma unroll 1
+    for (int q = 1; q < TW; ++q) {
+      dmax = fmax(dmax, tm.red[q][0]);
+      amax = fmax(amax, tm.red[q][1]);
     }
   }
   double vd = 0.0, va = 0.0;
@@ -1131,9 +1371,49 @@ __device__ __noinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T
   }
   out.ok = 1;
   out.drift = fmax(amax > 0.0 ? dmax / amax : 0.0, va > 0.0 ? vd / fmax(va, 1.0) : 0.0);
-  out.logdet = n * M.log_se2 + logdetC - lrs;
-  out.logL = -0.5 * (n * kLog2Pi + out.logdet + (yy - hv) / M.se2);
+  out.logdet = fma((double)n, M.log_se2, logdetC) - lrs;
+  out.logL = -0.5 * (fma((double)n, kLog2Pi, out.logdet) + (yy - hv) / M.se2);
   return out;
+}
+
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void team_refresh(const DevModel& M, const PeChain<T, BIG, L, MIX> W, const Lanes<L> ln) {
+  const PeTeam<typename PeTab<T>::C>& tm = pe_team<T>(M);
+  pe_refresh_part<T, BIG, L, MIX, kTeam>(M, W, tm.Cp, tm.ws, M.n_cap, tm.w, tm.wsq, tm.n, tm.N, ln);
+}
+// The rebuild as the chain's first warp calls it.
+template <typename T, bool BIG, int L, bool MIX, int TW>
+__device__ __forceinline__ RefreshOut pe_refresh(const DevModel& M, const PeChain<T, BIG, L, MIX> W, typename PeTab<T>::C* Cp,
+                                                 double* ws, int n_cap, const float* w, double wsq, int n, int N,
+                                                 const Lanes<L> ln) {
+  if constexpr (TW > 1) {
+    PeTeam<typename PeTab<T>::C>& tm = pe_team<T>(M);
+    if (ln.sl == 0) {
+      tm.op = kOpRefresh;
+      tm.Cp = Cp; tm.ws = ws; tm.w = w; tm.wsq = wsq; tm.n = n; tm.N = N;
+    }
+    team_bar();
+    const RefreshOut ro = pe_refresh_part<T, BIG, L, MIX, TW>(M, W, Cp, ws, n_cap, w, wsq, n, N, ln);
+    team_bar();
+    return ro;
+  } else {
+    return pe_refresh_part<T, BIG, L, MIX, 1>(M, W, Cp, ws, n_cap, w, wsq, n, N, ln);
+  }
+}
+// The other warps of a team, until the CTA has no chain left.
+template <typename T, bool BIG, int L, bool MIX>
+__device__ __noinline__ void team_help(const DevModel& M, const PeChain<T, BIG, L, MIX> W, const Lanes<L> ln) {
+  const PeTeam<typename PeTab<T>::C>& tm = pe_team<T>(M);
+  for (;;) {
+    team_bar();
+    const int op = tm.op;
+    if (op == kOpExit) return;
+    if (op == kOpScore) team_score<T, BIG, L, MIX>(M, W);
+    else if (op == kOpRows) team_rows<T, BIG, L, MIX>(M, W);
+    else if (op == kOpUpdate) team_update<T, BIG, L, MIX>(M, W);
+    else team_refresh<T, BIG, L, MIX>(M, W, ln);
+    team_bar();
+  }
 }
 
 // Scalars of an accepted move, from the proposal and its scoring.
@@ -1154,7 +1434,7 @@ template <typename C> struct AcceptOut {
 // Apply an accepted move to C^-1, v, y and the PE list. Returns the new N, and the new C^-1 storage
 // when it moves from the shared tile (capacity cap PEs) to the global slot (n_cap PEs). Inlined in
 // the step loop (the call's moves and the model constants' generic loads cost it 4 %).
-template <typename T, bool BIG, int L, bool MIX>
+template <typename T, bool BIG, int L, bool MIX, int TW>
 __device__ __forceinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevModel& M, const PeChain<T, BIG, L, MIX> W,
                                                                   typename PeTab<T>::C* Cp, int cap,
                                                                   typename PeTab<T>::C* Cg,
@@ -1182,6 +1462,7 @@ __device__ __forceinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevMo
   C* const uvd = W.ovb();  // u' / delta, once b is no longer read
   const T* const Vs = pe_V<T>();
   const unsigned short* const tij = pe_tij();
+  const bool team = TW > 1 && N > kSpecPes;  // the team's warps take part in the passes over C^-1
   C ig = czero<C>(), idl = czero<C>(), t = czero<C>(), fv = czero<C>(), nig = czero<C>();
   C bvf = czero<C>(), bk = czero<C>(), wk = czero<C>();
   if (has_p) {
@@ -1196,7 +1477,15 @@ __device__ __forceinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevMo
       }
     }
     csum2_m(bvf, bk, np, ln);
-    if constexpr (BIG) {
+    if (team) {
+      if constexpr (TW > 1) {
+        PeTeam<C>& tm = pe_team<T>(M);
+        if (ln.sl == 0) { tm.op = kOpRows; tm.Cp = Cp; tm.N = N; tm.np = np; }
+        team_bar();
+        team_rows<T, BIG, L, MIX>(M, W);
+        team_bar();
+      }
+    } else if constexpr (BIG) {
       __syncwarp(ln.gm);
 #pragma unroll 1
       for (int i = ln.sl; i < N; i += L) W.uv()[i] = dot_row4<C>(Cp, i, W.ovi(), W.ovb(), np);
@@ -1306,7 +1595,16 @@ __device__ __forceinline__ AcceptOut<typename PeTab<T>::C> pe_accept(const DevMo
   };
   TriWalk<L> tw;
   int e = ln.sl;
-  if constexpr (BIG) {
+  if (team) {
+    if constexpr (TW > 1) {
+      PeTeam<C>& tm = pe_team<T>(M);
+      if (ln.sl == 0) { tm.op = kOpUpdate; tm.Cp = Cp; tm.N = N; tm.jump = jump; tm.kk = kk; tm.nig = nig; tm.idl = idl; }
+      team_bar();
+      team_update<T, BIG, L, MIX>(M, W);
+      team_bar();
+      e = ne;
+    }
+  } else if constexpr (BIG) {
     // C^-1 in the global slot: four entries per lane and pass, all read before any is written
     // (each read is the entry itself or one in the unwritten last row), so that the loads of a
     // pass overlap
@@ -1387,7 +1685,7 @@ __device__ __noinline__ AcceptOut<typename PeTab<T>::C> pe_accept_call(const Dev
                                                                        typename PeTab<T>::C* Cg,
                                                                        const PeMove<typename PeTab<T>::C> mv, int n,
                                                                        int N, const Lanes<L> ln) {
-  return pe_accept<T, BIG, L, MIX>(M, W, Cp, cap, Cg, mv, n, N, ln);
+  return pe_accept<T, BIG, L, MIX, 1>(M, W, Cp, cap, Cg, mv, n, N, ln);
 }
 
 // The 2x2 algebra of Eqs. (16)-(18) in the scoring precision: log D, Delta nu and the status bits
@@ -1497,16 +1795,17 @@ __device__ __noinline__ void pe_hist_add(const PeChain<T, BIG, L, MIX> W, uint32
 // against 25.7; pile-up, 600 chains: 85.6 against 95.2) and leaves 255 registers. With two chains
 // per warp (L = 16) the half warps wait on each other, and 16 warps are better (30 000
 // low-occupancy chains: 31.5 ms, with 8 warps 42.9).
-constexpr int pe_min_ctas(int L) { return L == 16 ? 4 : 2; }
+constexpr int pe_min_ctas(int L, int TW) { return L == 16 || TW > 1 ? 4 : 2; }
 
-template <typename T, bool BIG, int L, bool MIX>
-__global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
+template <typename T, bool BIG, int L, bool MIX, int TW = 1>
+__global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L, TW))
     pe_kernel(const __grid_constant__ DevModel M, const __grid_constant__ BatchView B, const __grid_constant__ PeSlots G) {
   using C = typename PeTab<T>::C;
   constexpr bool fp32 = sizeof(T) == 4;
   const Lanes<L> ln = pe_lanes<L>();
   constexpr int kGroups = 32 / L;  // chains per warp
-  const int cw = (threadIdx.x >> 5) * kGroups + ln.g, nchains = (blockDim.x >> 5) * kGroups;
+  static_assert(TW == 1 || (TW == kTeam && L == 32), "a team is the CTA's warps");
+  const int cw = TW > 1 ? 0 : (threadIdx.x >> 5) * kGroups + ln.g, nchains = TW > 1 ? 1 : (blockDim.x >> 5) * kGroups;
   const int n_alloc = B.n_max, n_cap = M.n_cap, Ns = G.Ns;
   unsigned short* const tij = pe_tij();
   T* const Vs = pe_V<T>();
@@ -1532,7 +1831,13 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
   W.lb = (unsigned)a16(sizeof(int) * (size_t)n_cap);
   W.yb = (unsigned)a16(sizeof(T) * (size_t)n_alloc);
   W.pb = (unsigned)a16(sizeof(T) * (size_t)M.win_extra);
-  W.o = (unsigned)(pe_block_bytes<T>(M) + (size_t)cw * pe_chain_bytes<T, BIG, L, MIX>(n_cap, n_alloc, M.win_extra, Ns));
+  W.o = (unsigned)(pe_block_bytes<T>(M) + (TW > 1 ? kTeamBytes : 0u) + (size_t)cw * pe_chain_bytes<T, BIG, L, MIX>(n_cap, n_alloc, M.win_extra, Ns));
+  if constexpr (TW > 1) {
+    if (threadIdx.x >= 32) {
+      team_help<T, BIG, L, MIX>(M, W, ln);
+      return;
+    }
+  }
   PeStats& S = W.st();
   const size_t slot = (size_t)blockIdx.x * nchains + cw;
   int* const hist = G.hist + slot * (size_t)(n_cap + 1);
@@ -1648,7 +1953,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
         C qs = czero<C>();
         if constexpr (fp32) {
           // FP32 mode: the FP64 rebuild
-          const RefreshOut ro = pe_refresh<T, BIG, L, MIX>(M, W, Cp, ws, n_cap, w, S.wsq, n, ni, ln);
+          const RefreshOut ro = pe_refresh<T, BIG, L, MIX, TW>(M, W, Cp, ws, n_cap, w, S.wsq, n, ni, ln);
           ok = ro.ok != 0;
           if (ok && ln.sl == 0) { S.sum[PeStats::kLogdet] = ro.logdet; S.sum[PeStats::kLogL] = ro.logL; }
         } else {
@@ -2129,9 +2434,17 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
             for (int i = sp.ilo + ln.sl; i < sp.ihi; i += L) ayp += Vs[sp.ph + i * R] * W.y()[sp.w0 + i];
             C qp = czero<C>(), ck = czero<C>();
             T bvp = (T)0;
-            const int nt = tri(np);
+            const bool team = TW > 1 && np > kSpecPes;
+            const int nt = team ? 0 : tri(np);
             TriWalk<L> tw;
             int e = ln.sl;
+            if constexpr (TW > 1) {
+              if (team) {  // the helpers start; this warp's share comes after the sums below
+                PeTeam<C>& tm = pe_team<T>(M);
+                if (ln.sl == 0) { tm.op = kOpScore; tm.Cp = Cp; tm.np = np; }
+                team_bar();
+              }
+            }
             // the products of two entries e, e + L at a time (BIG, C^-1 in the global slot: two
             // such pairs, their loads ahead of their sums), added in order
             constexpr int PE = BIG ? 4 : 2;
@@ -2162,6 +2475,13 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
               const C ba = W.ovb()[a];
               bvp += (T)cnum(ba) * (T)cnum(W.v()[W.ovi()[a]]);
               if (opaque(jump == 2)) ck = cfma(Cp[pk(kk, W.ovi()[a])], ba, ck);
+            }
+            if constexpr (TW > 1) {
+              if (team) {
+                team_score<T, BIG, L, MIX>(M, W);
+                team_bar();
+                qp = pe_team<T>(M).part[ln.sl];
+              }
             }
             gsum4<L, L>(qp, ck, bvp, ayp, ln);
             const T bvT = bvp;  // b^T v at the scoring precision (the accept recomputes it)
@@ -2204,7 +2524,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
       // ---- accepted move: C^-1, v, y and the PE list
       if (apply) {
         {
-          const AcceptOut<C> ao = pe_accept<T, BIG, L, MIX>(M, W, Cp, cap, Cg, mv, n, N, ln);
+          const AcceptOut<C> ao = pe_accept<T, BIG, L, MIX, TW>(M, W, Cp, cap, Cg, mv, n, N, ln);
           Cp = ao.Cp;
           cap = ao.cap;
           N = ao.N;
@@ -2232,7 +2552,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
         set_summaries<MIX>(S, M.g, N, ms, c64(qs), inv1, ln.sl);
         __syncwarp(ln.gm);
         if (fp32 && M.refresh_every > 0 && S.n_acc_refresh >= M.refresh_every) {
-          const RefreshOut ro = pe_refresh<T, BIG, L, MIX>(M, W, Cp, ws, n_cap, w, S.wsq, n, N, ln);
+          const RefreshOut ro = pe_refresh<T, BIG, L, MIX, TW>(M, W, Cp, ws, n_cap, w, S.wsq, n, N, ln);
           C qr = czero<C>();
 #pragma unroll 1
           for (int i = ln.sl; i < N; i += L) qr = cadd(qr, W.v()[i]);
@@ -2270,7 +2590,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
     // ------------------------------------------------------------- chain end
     if (fp32 && M.refresh_every > 0 && S.n_acc_refresh > 0) {
       // the reported log-likelihood and log|Sigma| come from an FP64 rebuild
-      const RefreshOut ro = pe_refresh<T, BIG, L, MIX>(M, W, Cp, ws, n_cap, w, S.wsq, n, N, ln);
+      const RefreshOut ro = pe_refresh<T, BIG, L, MIX, TW>(M, W, Cp, ws, n_cap, w, S.wsq, n, N, ln);
       if (ln.sl == 0) {
         if (ro.ok) {
           S.sum[PeStats::kLogdet] = ro.logdet; S.sum[PeStats::kLogL] = ro.logL;
@@ -2317,6 +2637,10 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L))
     }
     __syncwarp(ln.gm);
   }
+  if constexpr (TW > 1) {
+    if (ln.sl == 0) pe_team<T>(M).op = kOpExit;
+    team_bar();
+  }
 }
 
 // Float-float copy of an FP64 table: hi = fl(x), lo = fl(x - hi).
@@ -2331,7 +2655,15 @@ __global__ void split_ff_kernel(const double* a, float* out, size_t n) {
 
 // The kernel instance for (precision, BIG, lanes) of a charge model; f receives its address.
 // The mixture has no BIG instance (its chains use the compact loops at any n_cap).
-template <bool MIX, typename F> cudaError_t with_pe_kernel(int precision, bool big, int lanes, F f) {
+template <bool MIX, typename F> cudaError_t with_pe_kernel(int precision, bool big, int lanes, bool team, F f) {
+  if (team) {
+    if (precision == FSMP_FP64 || lanes != 32) return cudaErrorInvalidValue;
+    if constexpr (MIX) {
+      return f(pe_kernel<float, false, 32, true, kTeam>);
+    } else {
+      return big ? f(pe_kernel<float, true, 32, false, kTeam>) : f(pe_kernel<float, false, 32, false, kTeam>);
+    }
+  }
   if constexpr (MIX) {
     if (precision == FSMP_FP64)
       return lanes == 16 ? f(pe_kernel<double, false, 16, true>) : f(pe_kernel<double, false, 32, true>);
@@ -2350,17 +2682,19 @@ template <bool MIX> cudaError_t pe_set_attributes(int precision, int max_smem) {
   for (int big = 0; big < (MIX ? 1 : 2); ++big)
     for (int lanes : {32, 16}) {
       if (big && lanes == 16) continue;
-      const cudaError_t e = with_pe_kernel<MIX>(precision, big != 0, lanes, [&](auto k) {
-        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-      });
-      if (e != cudaSuccess) return e;
+      for (int team = 0; team < (lanes == 32 && precision != FSMP_FP64 ? 2 : 1); ++team) {
+        const cudaError_t e = with_pe_kernel<MIX>(precision, big != 0, lanes, team != 0, [&](auto k) {
+          return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+        });
+        if (e != cudaSuccess) return e;
+      }
     }
   return cudaSuccess;
 }
 
-template <bool MIX> int pe_occupancy(int precision, int threads, size_t smem, bool big, int lanes) {
+template <bool MIX> int pe_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool team) {
   int n = 0;
-  const cudaError_t e = with_pe_kernel<MIX>(precision, big, lanes, [&](auto k) {
+  const cudaError_t e = with_pe_kernel<MIX>(precision, big, lanes, team, [&](auto k) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
   });
   return e == cudaSuccess ? n : 0;
@@ -2369,7 +2703,7 @@ template <bool MIX> int pe_occupancy(int precision, int threads, size_t smem, bo
 template <bool MIX>
 cudaError_t pe_launch(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                       void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                      bool big, cudaStream_t st) {
+                      bool big, bool team, cudaStream_t st) {
   PeSlots G;
   G.C = cinv;
   G.c_stride = c_stride;
@@ -2380,7 +2714,7 @@ cudaError_t pe_launch(const DevModel& M, const BatchView& B, int warps, int lane
   G.Ns = Ns;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  e = with_pe_kernel<MIX>(M.precision, big, lanes, [&](auto k) {
+  e = with_pe_kernel<MIX>(M.precision, big, lanes, team, [&](auto k) {
     k<<<ctas, warps * 32, smem, st>>>(M, B, G);
     return cudaSuccess;
   });

@@ -259,15 +259,17 @@ void CUDART_CB pack_done_cb(void* arg) {
 struct PeShape {
   int warps, tile, ctas;
   size_t smem;
+  bool team;
 };
 int pe_shape(const fsmp_ctx* c, int n_alloc, PeShape* s) {
+  s->team = false;
   const int tile = c->pe_tile_free ? std::min(c->p.n_cap, 32) : c->pe_tile;
   if (pe_limit_bytes(c->M, n_alloc, c->pe_warps, c->pe_lanes, tile) > (size_t)c->prop.sharedMemPerBlockOptin)
     return FSMP_ERR_INVALID;
   s->warps = c->pe_warps;
   s->tile = c->pe_tile;
   for (;;) {
-    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, s->tile);
+    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, s->tile, false);
     if (s->smem <= (size_t)c->prop.sharedMemPerBlockOptin) break;
     const bool slots = c->pe_c_stride > 0;  // room for C^-1 beyond the tile
     if (slots && s->tile > 16) s->tile = std::max(16, s->tile - 8);
@@ -276,11 +278,39 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, PeShape* s) {
     else return FSMP_ERR_INVALID;
   }
   int per_sm = pe_kernel_occupancy(c->p.precision, s->warps * 32, s->smem, pe_big(c->p.n_cap), c->pe_lanes,
-                                   c->M.n_comp > 1);
+                                   c->M.n_comp > 1, false);
   if (per_sm < 1) return FSMP_ERR_INVALID;
   if (c->p.pe_ctas_per_sm > 0) per_sm = std::min(per_sm, c->p.pe_ctas_per_sm);
   s->ctas = per_sm * c->prop.multiProcessorCount;
   return FSMP_OK;
+}
+
+// Teams: a CTA of four warps per chain, which work together on what a chain of more than 32 PEs does
+// with C^-1. A chain is then about three times as fast, but an SM holds 4 of them instead of 8, and
+// chains of few PEs get nothing from it. So teams serve launches that end with their longest
+// chains: up to 20 chains per SM (mixture, 1000 steps: 3000 chains 16.7 ms against 17.5 with a warp
+// per chain, 4000 chains 22.9 against 20.2; uneven windows: 3000 chains 16.4 ms against 24.7, 6000
+// chains 32.9 against 30.1), and up to 8 with the pile-up variant (1000 chains x 2000 steps 250 ms
+// against 600; 2000 chains x 300 steps 19.7 against 18.1). Only where the launch shape is left to
+// the library, and where a chain can have clearly more than 32 PEs.
+constexpr int kTeamChains = 20, kTeamChainsBig = 8;  // most chains per SM
+constexpr int kTeamMinCap = 64;                      // least capacity
+bool pe_team_shape(const fsmp_ctx* c, int n_alloc, int W, PeShape* s) {
+  const bool big = pe_big(c->p.n_cap);
+  if (c->p.threads_per_chain != 0 || c->p.pe_ctas_per_sm != 0 || !c->pe_tile_free || c->p.n_cap < kTeamMinCap ||
+      !pe_team_ok(c->p.precision, c->pe_lanes) || W > (big ? kTeamChainsBig : kTeamChains) * c->prop.multiProcessorCount)
+    return false;
+  PeShape t;
+  t.team = true;
+  t.warps = 4;
+  t.tile = c->pe_tile;  // 40; 96: a burst of 64 events 57 ms against 51, pile-up 245 against 255
+  t.smem = pe_smem_bytes(c->M, n_alloc, t.warps, c->pe_lanes, t.tile, true);
+  if (t.smem > (size_t)c->prop.sharedMemPerBlockOptin) return false;
+  const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, c->pe_lanes, c->M.n_comp > 1, true);
+  if (per_sm < 1) return false;
+  t.ctas = per_sm * c->prop.multiProcessorCount;
+  *s = t;
+  return true;
 }
 
 int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
@@ -288,11 +318,12 @@ int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
   PeShape s;
   if (pe_shape(c, B.n_max, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
-  const int cpc = s.warps * (32 / c->pe_lanes);
+  pe_team_shape(c, B.n_max, B.n_waveforms, &s);
+  const int cpc = s.team ? 1 : s.warps * (32 / c->pe_lanes);
   const int ctas = std::min(std::min(s.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
   const fsmp_ctx::PeSet& ps = c->pe_sets[set];
   cudaError_t e = launch_pe(c->M, B, s.warps, c->pe_lanes, ctas, s.tile, s.smem, ps.cinv, c->pe_c_stride,
-                            ps.ws, c->pe_ws_stride, ps.hist, ps.counter, st);
+                            ps.ws, c->pe_ws_stride, ps.hist, ps.counter, s.team, st);
   c->n_launches++;
   if (e != cudaSuccess) { set_error("launch_pe", cudaGetErrorString(e), __LINE__); return FSMP_ERR_CUDA; }
   return FSMP_OK;
