@@ -340,7 +340,7 @@ typedef struct {
  * batch laid out as for fsmp_run_device: time trial runs of its first `sample` waveforms for
  * `trial_steps` MCMC steps in each candidate shape -- lanes per chain (only if the context
  * was created with pe_lanes = 0), shared-memory tile of C^-1, warps per CTA and resident CTAs
- * per SM -- and keep the fastest for the context's later launches. The batch's own output and
+ * per SM, and a CTA of four warps per chain -- and keep the fastest for the context's later launches. The batch's own output and
  * trace buffers are not touched (the trials write to scratch). Later results do not depend on
  * the tile, warps or CTAs: a chain's arithmetic is the same in each. They do depend, up to
  * rounding, on the lane count; fix pe_lanes for results reproducible bit for bit.

@@ -123,6 +123,7 @@ struct fsmp_ctx {
   std::vector<PeSet> pe_sets;
   int pe_slots = 0, pe_warps = 4, pe_tile = 0, pe_lanes = 32;
   bool pe_lanes_free = false;  // pe_lanes left to fsmp_autotune
+  bool pe_team_always = false;  // fsmp_autotune found teams faster on its batch
   bool pe_tile_free = false;   // pe_tile neither given nor tuned
   size_t pe_c_stride = 0, pe_ws_stride = 0, pe_bytes = 0;
   std::atomic<long long> n_launches{0};  // chain-kernel launches
@@ -290,21 +291,27 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, PeShape* s) {
 // chains of few PEs get nothing from it. So teams serve launches that end with their longest
 // chains: up to 20 chains per SM (mixture, 1000 steps: 3000 chains 16.7 ms against 17.5 with a warp
 // per chain, 4000 chains 22.9 against 20.2; uneven windows: 3000 chains 16.4 ms against 24.7, 6000
-// chains 32.9 against 30.1), and up to 8 with the pile-up variant (1000 chains x 2000 steps 250 ms
-// against 600; 2000 chains x 300 steps 19.7 against 18.1). Only where the launch shape is left to
-// the library, and where a chain can have clearly more than 32 PEs.
+// chains 32.9 against 30.1). A pile-up chain is beyond 32 PEs for all but its first steps: there
+// teams serve any number of chains that run for 512 steps or more (6000 chains x 1000 steps: 398 ms
+// against 643, x 600 steps 174 against 212, x 300 steps 60 against 47), or start from a given state,
+// and up to 8 chains per SM otherwise (1000 chains x 500 steps 23 ms against 30). Only where the
+// launch shape is left to the library, and where a chain can have clearly more than 32 PEs.
 constexpr int kTeamChains = 20, kTeamChainsBig = 8;  // most chains per SM
+constexpr int kTeamStepsBig = 512;
 constexpr int kTeamMinCap = 64;                      // least capacity
-bool pe_team_shape(const fsmp_ctx* c, int n_alloc, int W, PeShape* s) {
+bool pe_team_shape(const fsmp_ctx* c, const BatchView& B, PeShape* s) {
   const bool big = pe_big(c->p.n_cap);
-  if (c->p.threads_per_chain != 0 || c->p.pe_ctas_per_sm != 0 || !c->pe_tile_free || c->p.n_cap < kTeamMinCap ||
-      !pe_team_ok(c->p.precision, c->pe_lanes) || W > (big ? kTeamChainsBig : kTeamChains) * c->prop.multiProcessorCount)
+  if (c->p.threads_per_chain != 0 || c->p.pe_ctas_per_sm != 0 || c->p.n_cap < kTeamMinCap ||
+      !pe_team_ok(c->p.precision, c->pe_lanes))
     return false;
+  const bool few = B.n_waveforms <= (big ? kTeamChainsBig : kTeamChains) * c->prop.multiProcessorCount;
+  const bool long_big = big && (B.z_init || (!B.n_steps_arr && B.n_steps >= kTeamStepsBig));
+  if (!c->pe_team_always && !(c->pe_tile_free && (few || long_big))) return false;
   PeShape t;
   t.team = true;
   t.warps = 4;
   t.tile = c->pe_tile;  // 40; 96: a burst of 64 events 57 ms against 51, pile-up 245 against 255
-  t.smem = pe_smem_bytes(c->M, n_alloc, t.warps, c->pe_lanes, t.tile, true);
+  t.smem = pe_smem_bytes(c->M, B.n_max, t.warps, c->pe_lanes, t.tile, true);
   if (t.smem > (size_t)c->prop.sharedMemPerBlockOptin) return false;
   const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, c->pe_lanes, c->M.n_comp > 1, true);
   if (per_sm < 1) return false;
@@ -318,7 +325,7 @@ int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
   PeShape s;
   if (pe_shape(c, B.n_max, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
-  pe_team_shape(c, B.n_max, B.n_waveforms, &s);
+  pe_team_shape(c, B, &s);
   const int cpc = s.team ? 1 : s.warps * (32 / c->pe_lanes);
   const int ctas = std::min(std::min(s.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
   const fsmp_ctx::PeSet& ps = c->pe_sets[set];
@@ -1145,7 +1152,8 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   const int set = (int)c->streams.size();
   const int tile0 = c->pe_tile, warps0 = c->pe_warps, ctas0 = c->p.pe_ctas_per_sm, lanes0 = c->pe_lanes;
   const bool tfree0 = c->pe_tile_free;
-  c->pe_tile_free = false;  // the trials run in the shapes they name, later launches in the chosen one
+  const bool team0 = c->pe_team_always;
+  c->pe_team_always = false;
   auto trial = [&](int lanes, int tile, int warps, int ctas, double* rate) -> int {
     c->pe_lanes = lanes; c->pe_tile = tile; c->pe_warps = warps; c->p.pe_ctas_per_sm = ctas;
     PeShape s;
@@ -1173,7 +1181,9 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   tiles.erase(std::unique(tiles.begin(), tiles.end()), tiles.end());
   double r0 = 0.0, best = -1.0;
   int bl = lanes0, bt = tile0, bw = warps0, bc = ctas0, n_tried = 0;
-  int rc = trial(lanes0, tile0, warps0, ctas0, &r0);
+  bool bteam = false;
+  int rc = trial(lanes0, tile0, warps0, ctas0, &r0);  // the default launch, a team per chain where its rule says so
+  c->pe_tile_free = false;  // the other trials run in the shapes they name, later launches in the chosen one
   if (rc == FSMP_OK) {
     best = r0; ++n_tried;
     // coordinate search: lanes per chain (when the context leaves it free), tile, warps per
@@ -1205,6 +1215,17 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
       ++n_tried;
       if (r > best) { best = r; bc = k; }
     }
+    // a team per chain, whatever the number of chains
+    if (rc == FSMP_OK && (lanes0 == 32 || c->pe_lanes_free)) {
+      double r;
+      c->pe_team_always = true;
+      rc = trial(32, tile0, warps0, ctas0, &r);
+      c->pe_team_always = false;
+      if (rc == FSMP_OK) {
+        ++n_tried;
+        if (r > best) { best = r; bteam = true; bl = 32; bt = tile0; bw = warps0; bc = ctas0; }
+      }
+    }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1212,11 +1233,14 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   if (rc != FSMP_OK) {
     c->pe_lanes = lanes0; c->pe_tile = tile0; c->pe_warps = warps0; c->p.pe_ctas_per_sm = ctas0;
     c->pe_tile_free = tfree0;
+    c->pe_team_always = team0;
     return rc;
   }
+  c->pe_team_always = bteam;
+  if (best == r0) c->pe_tile_free = tfree0;  // the default launch, with its rules
   c->pe_lanes = bl; c->pe_tile = bt; c->pe_warps = bw; c->p.pe_ctas_per_sm = bc;
   if (out) {
-    out->pe_tile = bt; out->chains_per_cta = bw * (32 / bl); out->ctas_per_sm = bc; out->n_tried = n_tried;
+    out->pe_tile = bt; out->chains_per_cta = bteam ? 1 : bw * (32 / bl); out->ctas_per_sm = bc; out->n_tried = n_tried;
     out->lanes_per_chain = bl;
     out->best_steps_per_s = best; out->default_steps_per_s = r0;
   }
