@@ -349,6 +349,20 @@ typedef struct {
  * bad arguments) or FSMP_ERR_CUDA / FSMP_ERR_NOMEM. */
 int fsmp_autotune(fsmp_ctx* ctx, const fsmp_device_batch* batch, int sample, int trial_steps, fsmp_tune* out);
 
+/* Shape of a PE-space launch. */
+typedef struct {
+  int lanes_per_chain;           /* 32 or 16                                                  */
+  int chains_per_cta;            /* 1 for a team                                              */
+  int pe_tile;                   /* PEs per chain whose C^-1 stays in shared memory           */
+  int ctas;                      /* CTAs launched                                             */
+  int team;                      /* 1: four warps of a CTA work on one chain                  */
+} fsmp_launch;
+
+/* The shape of the context's last PE-space launch (testing aid; results do not depend on it, but
+ * for lanes_per_chain). Call it once that launch has finished. FSMP_ERR_INVALID where the context
+ * has launched none. */
+int fsmp_last_launch(fsmp_ctx* ctx, fsmp_launch* out);
+
 /* fsmp_run_device for callers that cannot allocate device memory. The paper has no
  * counterpart: this is an integration aid. Some callers cannot call cudaMalloc -- code that
  * runs under a framework allocator owning all device memory, or in a service that forbids

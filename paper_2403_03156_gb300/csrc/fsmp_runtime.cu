@@ -128,6 +128,8 @@ struct fsmp_ctx {
   size_t pe_c_stride = 0, pe_ws_stride = 0, pe_bytes = 0;
   std::atomic<long long> n_launches{0};  // chain-kernel launches
   std::mutex tune_mu;                    // serialises fsmp_autotune calls
+  std::mutex launch_mu;                  // the last PE-space launch (fsmp_last_launch)
+  fsmp_launch last_launch{};             // (lanes_per_chain 0: none yet)
   // serving loop
   std::vector<cudaStream_t> streams;
   cudaStream_t gmem_stream = nullptr;
@@ -333,6 +335,8 @@ int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
                             ps.ws, c->pe_ws_stride, ps.hist, ps.counter, s.team, st);
   c->n_launches++;
   if (e != cudaSuccess) { set_error("launch_pe", cudaGetErrorString(e), __LINE__); return FSMP_ERR_CUDA; }
+  std::lock_guard<std::mutex> lk(c->launch_mu);
+  c->last_launch = fsmp_launch{c->pe_lanes, cpc, s.tile, ctas, s.team ? 1 : 0};
   return FSMP_OK;
 }
 
@@ -1261,6 +1265,15 @@ int fsmp_get_tables(fsmp_ctx* c, double* ser_out, int max_ser, int* ser_len, int
     if (phi_out) CK(cudaMemcpy(phi_out, c->phi + (d_lo + c->M.D), sizeof(double) * count, cudaMemcpyDeviceToHost));
     if (logphi_out) CK(cudaMemcpy(logphi_out, c->logphi + (d_lo + c->M.D), sizeof(double) * count, cudaMemcpyDeviceToHost));
   }
+  return FSMP_OK;
+}
+
+int fsmp_last_launch(fsmp_ctx* c, fsmp_launch* out) {
+  g_last_error[0] = 0;
+  if (!c || !out) return FSMP_ERR_INVALID;
+  std::lock_guard<std::mutex> lk(c->launch_mu);
+  if (c->last_launch.lanes_per_chain == 0) FAIL(FSMP_ERR_INVALID, "the context has made no PE-space launch");
+  *out = c->last_launch;
   return FSMP_OK;
 }
 

@@ -87,6 +87,11 @@ class Tune(ctypes.Structure):
                 ("lanes_per_chain", _c_int)]
 
 
+class Launch(ctypes.Structure):
+    _fields_ = [("lanes_per_chain", _c_int), ("chains_per_cta", _c_int), ("pe_tile", _c_int), ("ctas", _c_int),
+                ("team", _c_int)]
+
+
 class Info(ctypes.Structure):
     _fields_ = [("device", _c_int), ("sm_count", _c_int), ("smem_per_block_optin", _c_int),
                 ("ser_len", _c_int), ("R", _c_int), ("L_V", _c_int), ("n_smem_max", _c_int),
@@ -98,7 +103,7 @@ class Info(ctypes.Structure):
 EXPORTS = ["fsmp_create", "fsmp_submit", "fsmp_poll", "fsmp_destroy", "fsmp_run_device",
            "fsmp_get_tables", "fsmp_get_info", "fsmp_philox_blocks", "fsmp_strerror",
            "fsmp_last_error", "fsmp_measure_peaks", "fsmp_run_device_noalloc", "fsmp_autotune",
-           "fsmp_gelman_rubin", "fsmp_gelman_diag", "fsmp_lucyddm", "fsmp_lambda_mle"]
+           "fsmp_gelman_rubin", "fsmp_gelman_diag", "fsmp_lucyddm", "fsmp_lambda_mle", "fsmp_last_launch"]
 
 _lib = None
 
@@ -131,6 +136,7 @@ def load(build_if_missing: bool = False):
     L.fsmp_lucyddm.argtypes = [_vp, ctypes.POINTER(LucyBatch), _vp]
     L.fsmp_lambda_mle.argtypes = [_vp, _vp, _c_int, _c_int, _vp, _c_int, _vp]
     L.fsmp_get_tables.argtypes = [_vp, _vp, _c_int, ctypes.POINTER(_c_int), _c_int, _c_int, _vp, _vp]
+    L.fsmp_last_launch.argtypes = [_vp, ctypes.POINTER(Launch)]
     L.fsmp_get_info.argtypes = [_vp, ctypes.POINTER(Info)]
     L.fsmp_philox_blocks.argtypes = [_vp, ctypes.POINTER(_c_u64), _vp, _c_int, _vp]
     L.fsmp_measure_peaks.argtypes = [_vp, ctypes.POINTER(_c_double), ctypes.POINTER(_c_double),
@@ -377,6 +383,12 @@ class Context:
         d = {k: getattr(i, k) for k, _ in Info._fields_}
         d["name"] = i.name.decode()
         return d
+
+    def last_launch(self) -> dict:
+        """fsmp_last_launch: the shape of the last PE-space launch, once it has finished."""
+        s = Launch()
+        _check(load().fsmp_last_launch(self.h, ctypes.byref(s)), "fsmp_last_launch")
+        return {k: getattr(s, k) for k, _ in Launch._fields_}
 
     def measure_peaks(self) -> dict:
         a, b, c = _c_double(), _c_double(), _c_double()
