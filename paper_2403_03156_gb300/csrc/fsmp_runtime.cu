@@ -3,6 +3,7 @@
 // the serving loop (a scheduler thread that admits submitted requests by device memory,
 // packs them into persistent-kernel launches on a pool of streams, and hands finished
 // requests to fsmp_poll).
+#include <limits.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -255,16 +256,18 @@ void CUDART_CB pack_done_cb(void* arg) {
 }
 
 // ---- device batch from arrays already on the device
-// Launch shape of the PE-space kernel for windows up to n_alloc: warps per CTA, lanes per chain,
-// the shared tile of C^-1, and resident CTAs per SM from the hardware's occupancy rule. Where the
-// context's tile and warps do not fit shared memory (but are within its limits), a smaller tile (down to 16 PEs) and then fewer
-// warps are taken, and in the end a smaller tile still: the results do not depend on either.
+// Launch shape of the PE-space kernel for n_chains windows of up to n_alloc samples: warps per CTA,
+// lanes per chain, the shared tile of C^-1, and resident CTAs per SM from the hardware's occupancy
+// rule. Where the context's tile and warps do not fit shared memory (but are within its limits), a
+// smaller tile (down to 16 PEs) and then fewer warps are taken, and in the end a smaller tile still:
+// the results do not depend on either.
+constexpr int kTileSmall = 32;
 struct PeShape {
   int warps, tile, ctas;
   size_t smem;
   bool team;
 };
-int pe_shape(const fsmp_ctx* c, int n_alloc, PeShape* s) {
+int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
   s->team = false;
   const int tile = c->pe_tile_free ? std::min(c->p.n_cap, 32) : c->pe_tile;
   if (pe_limit_bytes(c->M, n_alloc, c->pe_warps, c->pe_lanes, tile) > (size_t)c->prop.sharedMemPerBlockOptin)
@@ -280,9 +283,22 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, PeShape* s) {
     else if (slots && s->tile > 0) s->tile = std::max(0, s->tile - 8);
     else return FSMP_ERR_INVALID;
   }
-  int per_sm = pe_kernel_occupancy(c->p.precision, s->warps * 32, s->smem, pe_big(c->p.n_cap), c->pe_lanes,
-                                   c->M.n_comp > 1, false);
+  auto occupancy = [&](size_t smem) {
+    return pe_kernel_occupancy(c->p.precision, s->warps * 32, smem, pe_big(c->p.n_cap), c->pe_lanes, c->M.n_comp > 1,
+                               false);
+  };
+  int per_sm = occupancy(s->smem);
   if (per_sm < 1) return FSMP_ERR_INVALID;
+  // The default tile (40) is 32 where that lets in another CTA that the launch has chains for: the 8
+  // KB more per CTA kept half of the chains out (pile-up model of 1024 samples, 2 CTAs per SM instead
+  // of 1: 6000 chains of 2 PEs x 300 steps 6.4 ms against 9.1, of 35 PEs 32.0 and 31.0; FP64, n_cap
+  // 128, windows of 400: 2000 chains of 15 PEs x 60 steps 4.8 and 5.2).
+  const int resident = per_sm * c->prop.multiProcessorCount * s->warps * (32 / c->pe_lanes);
+  if (c->pe_tile_free && c->pe_c_stride > 0 && s->tile > kTileSmall && n_chains > resident) {
+    const size_t smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, kTileSmall, false);
+    const int more = occupancy(smem);
+    if (more > per_sm) { per_sm = more; s->tile = kTileSmall; s->smem = smem; }
+  }
   if (c->p.pe_ctas_per_sm > 0) per_sm = std::min(per_sm, c->p.pe_ctas_per_sm);
   s->ctas = per_sm * c->prop.multiProcessorCount;
   return FSMP_OK;
@@ -326,7 +342,7 @@ int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   if (c->pe_sets.empty()) FAIL(FSMP_ERR_INVALID, "the PE-space kernel was not set up at fsmp_create");
   if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
   PeShape s;
-  if (pe_shape(c, B.n_max, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
+  if (pe_shape(c, B.n_max, B.n_waveforms, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
   pe_team_shape(c, B, &s);
   const int cpc = s.team ? 1 : s.warps * (32 / c->pe_lanes);
   const int ctas = std::min(std::min(s.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
@@ -974,7 +990,7 @@ int fsmp_create(const fsmp_params* params, fsmp_ctx** out) {
       c->pe_lanes = lanes;
       for (int nn : {std::min(64, p.n_max), p.n_max}) {
         PeShape s;
-        if (pe_shape(c.get(), nn, &s) == FSMP_OK) slots = std::max(slots, s.ctas * s.warps * (32 / lanes));
+        if (pe_shape(c.get(), nn, INT_MAX, &s) == FSMP_OK) slots = std::max(slots, s.ctas * s.warps * (32 / lanes));
       }
     }
     c->pe_lanes = lanes0;
@@ -1161,7 +1177,8 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   auto trial = [&](int lanes, int tile, int warps, int ctas, double* rate) -> int {
     c->pe_lanes = lanes; c->pe_tile = tile; c->pe_warps = warps; c->p.pe_ctas_per_sm = ctas;
     PeShape s;
-    if (pe_shape(c, B.n_max, &s) != FSMP_OK || s.warps != warps || s.tile != tile) { *rate = -1.0; return FSMP_OK; }
+    // (the default shape, timed first, is taken as pe_shape makes it)
+    if (pe_shape(c, B.n_max, B.n_waveforms, &s) != FSMP_OK || (!c->pe_tile_free && (s.warps != warps || s.tile != tile))) { *rate = -1.0; return FSMP_OK; }
     float best_ms = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {  // the first run warms the caches and the code
       if (cudaEventRecord(e0, st) != cudaSuccess) return FSMP_ERR_CUDA;
@@ -1289,7 +1306,7 @@ int fsmp_get_info(fsmp_ctx* c, fsmp_info* o) {
   o->n_smem_max = c->n_smem_max;
   if (c->p.kernel == FSMP_KERNEL_PE) {  // pe_lanes lanes per chain, pe_warps warps per CTA
     PeShape s;
-    if (pe_shape(c, c->p.n_max, &s) == FSMP_OK) {
+    if (pe_shape(c, c->p.n_max, INT_MAX, &s) == FSMP_OK) {
       o->threads_per_chain = c->pe_lanes;
       o->ctas_per_sm = s.ctas / c->prop.multiProcessorCount;
     }
