@@ -635,10 +635,16 @@ struct PeStats {
 // lanes' partial sums in the same order (each of its lanes holds kSpec of them). Four steps: with
 // eight the batch's loops are twice as long, and wait for instructions too (low occupancy 106 ms
 // against 104, one event 5.97 against 5.22). Up to 32 PEs: beyond, the entries scored for steps
-// that do not count cost what the batch saves. 20 000 uneven windows x 2000 steps: 120 -> 110 ms,
-// 100 000 low-occupancy chains x 1000: 134 -> 103 ms, 256 FP64 chains x 1000: 13.7 -> 9.8 ms.
+// that do not count cost what the batch saves. In FP64 mode, where the entries' pair arithmetic is
+// most of a step, that is so from 8 PEs on with 32 lanes and from 12 on with 16 (608 chains of 24 PEs
+// x 150 steps: 6.9 ms with batches up to 32 PEs, 5.8 up to 8; of 8 PEs 5.2 and 4.3; with batches up
+// to 4, 2000 chains of 2 PEs take 6.3 instead of 5.8). 20 000 uneven windows x 2000 steps: 120 -> 110
+// ms, 100 000 low-occupancy chains x 1000: 134 -> 103 ms, 256 FP64 chains x 1000: 13.7 -> 9.8 ms.
 constexpr int kSpec = kSub;
 constexpr int kSpecPes = 32;   // most PEs of a chain scored this way (indices in W.ix())
+template <typename T> __host__ __device__ constexpr int spec_pes(int L) {
+  return sizeof(T) == 4 ? kSpecPes : (L == 32 ? 8 : 12);
+}
 constexpr int kCounts = 8;     // integer counts of a chain, per subgroup (PeChain::cnt)
 
 // A step's addition to count q: sums over the samples after burn-in of N, N^2, k0 and k0^2, the
@@ -2068,7 +2074,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L, TW))
       bool one = true;         // that step is still to be counted
       unsigned words = 0;
       int last;
-      if (!BIG && N <= kSpecPes) {
+      if (!BIG && N <= spec_pes<T>(L)) {
         // ---------------------------------------------- a batch of steps, one per subgroup
         constexpr int gw = L / kSpec;  // lanes of a subgroup
         const int gi = ln.sl / gw, m = ln.sl % gw;
