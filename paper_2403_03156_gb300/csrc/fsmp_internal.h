@@ -280,7 +280,10 @@ cudaError_t measure_peaks(int sm_count, double* smem_gbs, double* fp64_tflops, d
 // per CTA with windows up to n_alloc and a shared tile of C^-1 for Ns PEs per chain; FP64
 // workspace doubles per chain slot (FP32 mode); entries of a global C^-1 slot; ints of an N
 // histogram slot.
-size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns, bool team);
+// The forms of the PE-space kernel: a warp (or half warp) per chain; the same with room for more
+// CTAs on an SM (mixture only, see pe_min_ctas); a team of four warps per chain.
+enum PeForm { kPeWarp = 0, kPeWarpMore = 1, kPeTeam = 2 };
+size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns, PeForm form);
 size_t pe_limit_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns);
 size_t pe_ws_slot_doubles(int n_cap);
 size_t pe_c_entries(int n_cap);  // entries of a global C^-1 slot (packed triangle)
@@ -288,23 +291,25 @@ size_t pe_c_entry_bytes(int precision);  // bytes of one C^-1 entry (a pair of F
 inline size_t pe_hist_ints(int n_cap) { return (size_t)n_cap + 1; }
 cudaError_t pe_kernel_attributes(int precision, int max_smem);
 cudaError_t launch_split_ff(const double* a, float* out, size_t n, cudaStream_t st);
-int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool mix, bool team);
+int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool mix, PeForm form);
 // The MCP-mixture instances (fsmp_pe_mix.cu); launch_pe dispatches to them when M.n_comp > 1.
 cudaError_t pe_mix_attributes(int precision, int max_smem);
-int pe_mix_occupancy(int precision, int threads, size_t smem, int lanes, bool team);
+int pe_mix_occupancy(int precision, int threads, size_t smem, int lanes, PeForm form);
 cudaError_t pe_mix_launch(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                           void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                          bool team, cudaStream_t st);
+                          PeForm form, cudaStream_t st);
 bool pe_big(int n_cap);
 // A team (4 warps, one CTA) per chain: FP32 mode, 32 lanes; warps is 4 then.
 bool pe_team_ok(int precision, int lanes);
+// The form with more CTAs exists: the mixture in FP32 mode, 32 lanes.
+bool pe_more_ok(const DevModel& M, int lanes);
 bool pe_lanes_ok(int lanes, int n_cap);
 // Slots (C^-1, workspace, histogram) are indexed by resident chain: CTA x warps x (32 / lanes) (a
 // team: CTA).
 // counter: one int of device memory, zeroed on `st` before the launch.
 cudaError_t launch_pe(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                       void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                      bool team, cudaStream_t st);
+                      PeForm form, cudaStream_t st);
 // lambda_FSMP of n_hist histograms of n_max + 1 counts on `lanes` (32 or 16) lanes each, by the
 // device function the chain kernels end with (testing aid; fsmp_pe.cu).
 cudaError_t launch_lambda_mle(const int* h, int n_hist, int n_max, const double* lambda0, double* out, int lanes,

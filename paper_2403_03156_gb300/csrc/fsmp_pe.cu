@@ -6,9 +6,9 @@
 
 namespace fsmp {
 
-size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns, bool team) {
-  const int chains = team ? 1 : warps * (32 / lanes);
-  const size_t cmd = team ? kTeamBytes : 0;
+size_t pe_smem_bytes(const DevModel& M, int n_alloc, int warps, int lanes, int Ns, PeForm form) {
+  const int chains = form == kPeTeam ? 1 : warps * (32 / lanes);
+  const size_t cmd = form == kPeTeam ? kTeamBytes : 0;
   auto bytes = [&](auto big, auto lane_count, auto mix) {
     constexpr bool BIG = decltype(big)::value, MIX = decltype(mix)::value;
     constexpr int L = decltype(lane_count)::value;
@@ -61,16 +61,16 @@ bool pe_big(int n_cap) { return n_cap > 192; }
 bool pe_lanes_ok(int lanes, int n_cap) { return lanes == 32 || (lanes == 16 && !pe_big(n_cap)); }
 
 bool pe_team_ok(int precision, int lanes) { return precision != FSMP_FP64 && lanes == 32; }
-
+bool pe_more_ok(const DevModel& M, int lanes) { return M.n_comp > 1 && M.precision != FSMP_FP64 && lanes == 32; }
 
 cudaError_t pe_kernel_attributes(int precision, int max_smem) {
   const cudaError_t e = pe_set_attributes<false>(precision, max_smem);
   return e != cudaSuccess ? e : pe_mix_attributes(precision, max_smem);
 }
 
-int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool mix, bool team) {
-  if (mix) return pe_mix_occupancy(precision, threads, smem, lanes, team);
-  return pe_occupancy<false>(precision, threads, smem, big, lanes, team);
+int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool mix, PeForm form) {
+  if (mix) return pe_mix_occupancy(precision, threads, smem, lanes, form);
+  return pe_occupancy<false>(precision, threads, smem, big, lanes, form);
 }
 
 // lambda_FSMP of given N histograms (testing aid): the device function every chain ends with,
@@ -97,14 +97,15 @@ cudaError_t launch_lambda_mle(const int* h, int n_hist, int n_max, const double*
 
 cudaError_t launch_pe(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                       void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                      bool team, cudaStream_t st) {
+                      PeForm form, cudaStream_t st) {
   if (hist == nullptr || !pe_lanes_ok(lanes, M.n_cap)) return cudaErrorInvalidValue;
-  if (team && (!pe_team_ok(M.precision, lanes) || warps != kTeam)) return cudaErrorInvalidValue;
+  if (form == kPeTeam && (!pe_team_ok(M.precision, lanes) || warps != kTeam)) return cudaErrorInvalidValue;
+  if (form == kPeWarpMore && !pe_more_ok(M, lanes)) return cudaErrorInvalidValue;
   if (M.n_comp > 1)
-    return pe_mix_launch(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter, team,
+    return pe_mix_launch(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter, form,
                          st);
   return pe_launch<false>(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter,
-                          pe_big(M.n_cap), team, st);
+                          pe_big(M.n_cap), form, st);
 }
 
 }  // namespace fsmp

@@ -1801,10 +1801,17 @@ __device__ __noinline__ void pe_hist_add(const PeChain<T, BIG, L, MIX> W, uint32
 // against 25.7; pile-up, 600 chains: 85.6 against 95.2) and leaves 255 registers. With two chains
 // per warp (L = 16) the half warps wait on each other, and 16 warps are better (30 000
 // low-occupancy chains: 31.5 ms, with 8 warps 42.9).
-constexpr int pe_min_ctas(int L, int TW) { return L == 16 || TW > 1 ? 4 : 2; }
+//
+// The mixture's FP32 instance takes 180 registers, so 2 CTAs (8 warps); the dynode one 168 and 3. Its
+// chains of more than 40 PEs gain from the L1 that 2 CTAs leave (608 of 50 PEs x 600 steps: 9.7 ms
+// against 13.6 with 3 CTAs, 5000 of 0.5 to 50 PEs 11.4 against 13.9), but where an SM has enough
+// light chains, 12 warps do more steps than 8: so it comes in both (MORE: 170 registers, 3 CTAs;
+// 16 000 chains: 2 PEs 16.2 -> 13.2 ms, 8 PEs 27.9 -> 23.7, 24 PEs 62.9 -> 58.9, 0.5 to 50 33.6 ->
+// 30.9; n_cap 48, 6000 of 16 PEs 17.2 -> 15.2).
+constexpr int pe_min_ctas(int L, int TW, bool MORE) { return L == 16 || TW > 1 ? 4 : (MORE ? 3 : 2); }
 
-template <typename T, bool BIG, int L, bool MIX, int TW = 1>
-__global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L, TW))
+template <typename T, bool BIG, int L, bool MIX, int TW = 1, bool MORE = false>
+__global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L, TW, MORE))
     pe_kernel(const __grid_constant__ DevModel M, const __grid_constant__ BatchView B, const __grid_constant__ PeSlots G) {
   using C = typename PeTab<T>::C;
   constexpr bool fp32 = sizeof(T) == 4;
@@ -2661,14 +2668,20 @@ __global__ void split_ff_kernel(const double* a, float* out, size_t n) {
 
 // The kernel instance for (precision, BIG, lanes) of a charge model; f receives its address.
 // The mixture has no BIG instance (its chains use the compact loops at any n_cap).
-template <bool MIX, typename F> cudaError_t with_pe_kernel(int precision, bool big, int lanes, bool team, F f) {
-  if (team) {
+template <bool MIX, typename F> cudaError_t with_pe_kernel(int precision, bool big, int lanes, PeForm form, F f) {
+  if (form == kPeTeam) {
     if (precision == FSMP_FP64 || lanes != 32) return cudaErrorInvalidValue;
     if constexpr (MIX) {
       return f(pe_kernel<float, false, 32, true, kTeam>);
     } else {
       return big ? f(pe_kernel<float, true, 32, false, kTeam>) : f(pe_kernel<float, false, 32, false, kTeam>);
     }
+  }
+  if (form == kPeWarpMore) {
+    if constexpr (MIX) {
+      if (precision != FSMP_FP64 && lanes == 32) return f(pe_kernel<float, false, 32, true, 1, true>);
+    }
+    return cudaErrorInvalidValue;
   }
   if constexpr (MIX) {
     if (precision == FSMP_FP64)
@@ -2688,8 +2701,10 @@ template <bool MIX> cudaError_t pe_set_attributes(int precision, int max_smem) {
   for (int big = 0; big < (MIX ? 1 : 2); ++big)
     for (int lanes : {32, 16}) {
       if (big && lanes == 16) continue;
-      for (int team = 0; team < (lanes == 32 && precision != FSMP_FP64 ? 2 : 1); ++team) {
-        const cudaError_t e = with_pe_kernel<MIX>(precision, big != 0, lanes, team != 0, [&](auto k) {
+      for (PeForm form : {kPeWarp, kPeWarpMore, kPeTeam}) {
+        if (form != kPeWarp && (lanes != 32 || precision == FSMP_FP64)) continue;
+        if (form == kPeWarpMore && !MIX) continue;
+        const cudaError_t e = with_pe_kernel<MIX>(precision, big != 0, lanes, form, [&](auto k) {
           return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         });
         if (e != cudaSuccess) return e;
@@ -2698,9 +2713,9 @@ template <bool MIX> cudaError_t pe_set_attributes(int precision, int max_smem) {
   return cudaSuccess;
 }
 
-template <bool MIX> int pe_occupancy(int precision, int threads, size_t smem, bool big, int lanes, bool team) {
+template <bool MIX> int pe_occupancy(int precision, int threads, size_t smem, bool big, int lanes, PeForm form) {
   int n = 0;
-  const cudaError_t e = with_pe_kernel<MIX>(precision, big, lanes, team, [&](auto k) {
+  const cudaError_t e = with_pe_kernel<MIX>(precision, big, lanes, form, [&](auto k) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
   });
   return e == cudaSuccess ? n : 0;
@@ -2709,7 +2724,7 @@ template <bool MIX> int pe_occupancy(int precision, int threads, size_t smem, bo
 template <bool MIX>
 cudaError_t pe_launch(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                       void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                      bool big, bool team, cudaStream_t st) {
+                      bool big, PeForm form, cudaStream_t st) {
   PeSlots G;
   G.C = cinv;
   G.c_stride = c_stride;
@@ -2720,7 +2735,7 @@ cudaError_t pe_launch(const DevModel& M, const BatchView& B, int warps, int lane
   G.Ns = Ns;
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  e = with_pe_kernel<MIX>(M.precision, big, lanes, team, [&](auto k) {
+  e = with_pe_kernel<MIX>(M.precision, big, lanes, form, [&](auto k) {
     k<<<ctas, warps * 32, smem, st>>>(M, B, G);
     return cudaSuccess;
   });

@@ -7,15 +7,15 @@ namespace fsmp {
 
 cudaError_t pe_mix_attributes(int precision, int max_smem) { return pe_set_attributes<true>(precision, max_smem); }
 
-int pe_mix_occupancy(int precision, int threads, size_t smem, int lanes, bool team) {
-  return pe_occupancy<true>(precision, threads, smem, false, lanes, team);
+int pe_mix_occupancy(int precision, int threads, size_t smem, int lanes, PeForm form) {
+  return pe_occupancy<true>(precision, threads, smem, false, lanes, form);
 }
 
 cudaError_t pe_mix_launch(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                           void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
-                          bool team, cudaStream_t st) {
+                          PeForm form, cudaStream_t st) {
   return pe_launch<true>(M, B, warps, lanes, ctas, Ns, smem, cinv, c_stride, ws, ws_stride, hist, counter, false,
-                         team, st);
+                         form, st);
 }
 
 }  // namespace fsmp

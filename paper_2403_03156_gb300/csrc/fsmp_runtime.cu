@@ -265,17 +265,24 @@ constexpr int kTileSmall = 32;
 struct PeShape {
   int warps, tile, ctas;
   size_t smem;
-  bool team;
+  PeForm form;
 };
+// The mixture's form with more CTAs per SM (see pe_min_ctas): for launches that fill the SMs
+// many times over, and where no chain goes far beyond the tile. (With n_cap 128, 2000 to 6000 chains
+// of 2 to 32 PEs are 0 to 24 % faster in it, of 0.5 to 50 PEs 15 to 30 % slower.)
+constexpr int kMoreChains = 40;  // chains per SM
+constexpr int kMoreCap = 64;     // n_cap below
 int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
-  s->team = false;
+  const bool many = n_chains > kMoreChains * c->prop.multiProcessorCount || c->p.n_cap < kMoreCap;
+  const bool more = pe_more_ok(c->M, c->pe_lanes) && (c->p.pe_ctas_per_sm > 0 ? c->p.pe_ctas_per_sm > 2 : many);
+  s->form = more ? kPeWarpMore : kPeWarp;
   const int tile = c->pe_tile_free ? std::min(c->p.n_cap, 32) : c->pe_tile;
   if (pe_limit_bytes(c->M, n_alloc, c->pe_warps, c->pe_lanes, tile) > (size_t)c->prop.sharedMemPerBlockOptin)
     return FSMP_ERR_INVALID;
   s->warps = c->pe_warps;
   s->tile = c->pe_tile;
   for (;;) {
-    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, s->tile, false);
+    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, s->tile, s->form);
     if (s->smem <= (size_t)c->prop.sharedMemPerBlockOptin) break;
     const bool slots = c->pe_c_stride > 0;  // room for C^-1 beyond the tile
     if (slots && s->tile > 16) s->tile = std::max(16, s->tile - 8);
@@ -285,7 +292,7 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
   }
   auto occupancy = [&](size_t smem) {
     return pe_kernel_occupancy(c->p.precision, s->warps * 32, smem, pe_big(c->p.n_cap), c->pe_lanes, c->M.n_comp > 1,
-                               false);
+                               s->form);
   };
   int per_sm = occupancy(s->smem);
   if (per_sm < 1) return FSMP_ERR_INVALID;
@@ -295,7 +302,7 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
   // 128, windows of 400: 2000 chains of 15 PEs x 60 steps 4.8 and 5.2).
   const int resident = per_sm * c->prop.multiProcessorCount * s->warps * (32 / c->pe_lanes);
   if (c->pe_tile_free && c->pe_c_stride > 0 && s->tile > kTileSmall && n_chains > resident) {
-    const size_t smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, kTileSmall, false);
+    const size_t smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, kTileSmall, s->form);
     const int more = occupancy(smem);
     if (more > per_sm) { per_sm = more; s->tile = kTileSmall; s->smem = smem; }
   }
@@ -326,12 +333,12 @@ bool pe_team_shape(const fsmp_ctx* c, const BatchView& B, PeShape* s) {
   const bool long_big = big && (B.z_init || (!B.n_steps_arr && B.n_steps >= kTeamStepsBig));
   if (!c->pe_team_always && !(c->pe_tile_free && (few || long_big))) return false;
   PeShape t;
-  t.team = true;
+  t.form = kPeTeam;
   t.warps = 4;
   t.tile = c->pe_tile;  // 40; 96: a burst of 64 events 57 ms against 51, pile-up 245 against 255
-  t.smem = pe_smem_bytes(c->M, B.n_max, t.warps, c->pe_lanes, t.tile, true);
+  t.smem = pe_smem_bytes(c->M, B.n_max, t.warps, c->pe_lanes, t.tile, t.form);
   if (t.smem > (size_t)c->prop.sharedMemPerBlockOptin) return false;
-  const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, c->pe_lanes, c->M.n_comp > 1, true);
+  const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, c->pe_lanes, c->M.n_comp > 1, t.form);
   if (per_sm < 1) return false;
   t.ctas = per_sm * c->prop.multiProcessorCount;
   *s = t;
@@ -344,15 +351,16 @@ int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   PeShape s;
   if (pe_shape(c, B.n_max, B.n_waveforms, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
   pe_team_shape(c, B, &s);
-  const int cpc = s.team ? 1 : s.warps * (32 / c->pe_lanes);
+  const bool team = s.form == kPeTeam;
+  const int cpc = team ? 1 : s.warps * (32 / c->pe_lanes);
   const int ctas = std::min(std::min(s.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
   const fsmp_ctx::PeSet& ps = c->pe_sets[set];
   cudaError_t e = launch_pe(c->M, B, s.warps, c->pe_lanes, ctas, s.tile, s.smem, ps.cinv, c->pe_c_stride,
-                            ps.ws, c->pe_ws_stride, ps.hist, ps.counter, s.team, st);
+                            ps.ws, c->pe_ws_stride, ps.hist, ps.counter, s.form, st);
   c->n_launches++;
   if (e != cudaSuccess) { set_error("launch_pe", cudaGetErrorString(e), __LINE__); return FSMP_ERR_CUDA; }
   std::lock_guard<std::mutex> lk(c->launch_mu);
-  c->last_launch = fsmp_launch{c->pe_lanes, cpc, s.tile, ctas, s.team ? 1 : 0};
+  c->last_launch = fsmp_launch{c->pe_lanes, cpc, s.tile, ctas, team ? 1 : 0};
   return FSMP_OK;
 }
 

@@ -1,5 +1,6 @@
 """The default launch shape holds as many chains on an SM as the smaller tile of C^-1 (32 PEs)
 allows: a larger tile is for contexts where it takes no chain's place."""
+import numpy as np
 import pytest
 
 from paper_2403_03156_gb300 import fsmp, workloads
@@ -17,3 +18,27 @@ def test_the_default_tile_keeps_no_chain_out(workload, n_cap, n_max, precision):
     p = dict(workloads.CONFIGS[workload]["params"], n_cap=n_cap, n_max=n_max, precision=precision, n_streams=1)
     with gpu_util.context(p) as free, gpu_util.context(dict(p, pe_tile=32)) as small:
         assert free.info()["ctas_per_sm"] >= small.info()["ctas_per_sm"] >= 1
+
+
+@pytest.mark.parametrize("n_cap,n_waveforms,per_sm", [(128, 7000, 3), (48, 2000, 3), (128, 3500, 2)])
+def test_mixture_chains_per_sm(n_cap, n_waveforms, per_sm):
+    """Three CTAs of mixture chains on an SM where the launch fills the SMs many times over or n_cap is
+    small, else two; their outputs are the same bit for bit."""
+    torch = pytest.importorskip("torch")
+    dev = torch.device("cuda", 0)
+    cfg = workloads.CONFIGS["mcp_uneven_20k"]
+    p = dict(cfg["params"], n_cap=n_cap, n_max=512, precision=fsmp.FP32_REFRESH, refresh_every=16, pe_lanes=32, n_streams=1)
+    rng = np.random.Generator(np.random.PCG64(23))
+    b, _ = workloads.simulate(p, np.geomspace(50.0 if n_cap > 100 else 20.0, 0.5, n_waveforms), rng.uniform(30, 40, n_waveforms), rng, "trimmed")
+    got = []
+    for shape in (dict(threads_per_chain=128), dict(pe_ctas_per_sm=2), dict(pe_ctas_per_sm=3)):
+        d = {k: torch.from_numpy(np.ascontiguousarray(b[k])).to(dev) for k in ("samples", "offsets", "lambda0", "t_origin_ns")}
+        d["out"] = torch.zeros(n_waveforms * fsmp.SUMMARY_DTYPE.itemsize, dtype=torch.uint8, device=dev)
+        with gpu_util.context(dict(p, **shape)) as ctx:
+            ctx.run_device(d, n_steps=120, burn_in=20, seed=9, n_max_hint=512)
+            torch.cuda.synchronize(dev)
+            ctas = ctx.last_launch()["ctas"]
+            assert ctas == ctx.info()["sm_count"] * shape.get("pe_ctas_per_sm", per_sm)
+        got.append(d["out"].cpu().numpy())
+    for other in got[1:]:
+        np.testing.assert_array_equal(got[0], other)
