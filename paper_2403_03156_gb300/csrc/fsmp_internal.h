@@ -306,10 +306,15 @@ bool pe_more_ok(const DevModel& M, int lanes);
 bool pe_lanes_ok(int lanes, int n_cap);
 // Slots (C^-1, workspace, histogram) are indexed by resident chain: CTA x warps x (32 / lanes) (a
 // team: CTA).
-// counter: one int of device memory, zeroed on `st` before the launch.
+// counter: one int of device memory that the caller sets to 0 on `st` before the launch (or to
+// B.n_waveforms: then the launch runs no chain).
 cudaError_t launch_pe(const DevModel& M, const BatchView& B, int warps, int lanes, int ctas, int Ns, size_t smem,
                       void* cinv, size_t c_stride, double* ws, size_t ws_stride, int* hist, int* counter,
                       PeForm form, cudaStream_t st);
+// Chooses the form of a launch that is made in both, a warp and a team per chain, by the estimated
+// time of each on `sms` SMs: sets the chain counter of the chosen form (counters[0] a warp per
+// chain, counters[1] a team) to 0, the other's to n_waveforms, and counters[2] to 1 for teams.
+cudaError_t launch_pe_form(const DevModel& M, const BatchView& B, int sms, int* counters, cudaStream_t st);
 // lambda_FSMP of n_hist histograms of n_max + 1 counts on `lanes` (32 or 16) lanes each, by the
 // device function the chain kernels end with (testing aid; fsmp_pe.cu).
 cudaError_t launch_lambda_mle(const int* h, int n_hist, int n_max, const double* lambda0, double* out, int lanes,

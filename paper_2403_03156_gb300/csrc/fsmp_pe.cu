@@ -73,6 +73,95 @@ int pe_kernel_occupancy(int precision, int threads, size_t smem, bool big, int l
   return pe_occupancy<false>(precision, threads, smem, big, lanes, form);
 }
 
+// ---- a warp or a team per chain, by the chains' expected PEs
+//
+// A team makes a chain of many PEs two to three times as fast, but an SM holds 4 teams where it
+// holds 8 to 12 warps with a chain each, and chains of up to 32 PEs get nothing from it. So a launch
+// that ends with its longest chains is faster in teams and one that ends when the SMs have worked
+// through all chains is slower (uneven windows x 600 steps, ms with a warp and with a team per chain:
+// 3040 chains of lambda0 0.5 to 50: 13.4, 10.6; of 0.5 to 25: 6.5, 7.7; all of 8: 5.1, 9.0; 1216 of
+// 0.5 to 50: 11.9, 6.6; all of 8: 3.1, 4.3; pile-up model, 1216 of 0.5 to 200: 47.4, 22.5; of 5: 3.3,
+// 5.2). Which of the two a launch is depends
+// on its lambda0 and steps, which are on the device: this kernel estimates both times and sets the
+// chain counters so that only the faster form's launch finds chains (the other's ends at once: 3 us
+// and this kernel's 3 us).
+//
+// The estimate: a chain starts empty (or from n_init PEs) and moves towards lambda0 by 0.22 PEs a
+// step. Its step costs a polynomial in its PEs: `lat` us on its own, `thr` us of an SM that is full.
+// A launch takes the longest chain's time or the SMs' share of all chains, whichever is longer (a
+// smooth maximum). Fitted to 404 timed pairs of launches: lambda0 from 1 to 200, alone and mixed,
+// 152 to 6000 chains, 150 to 1500 steps. Of the 276 with more than 608 chains it takes the slower
+// form 13 times, by more than 10 % five times.
+constexpr float kGrowth = 0.22f;  // PEs a step
+struct FormCost {
+  float lat[4], thr[4];
+};
+constexpr FormCost kCost[2][2] = {
+    // n_cap <= 192: a warp per chain, a team
+    {{{2.1f, 0.22f, 4.3e-3f, 4.1e-5f}, {0.17f, 0.036f, 2.8e-4f, 3.7e-6f}},
+     {{3.1f, 0.18f, 5.5e-4f, 1.8e-7f}, {0.27f, 0.068f, 7.1e-5f, 1.0e-7f}}},
+    // above
+    {{{2.8f, 0.24f, 8.4e-3f, 1.2e-6f}, {0.26f, 0.076f, 1.2e-4f, 4.1e-6f}},
+     {{4.9f, 0.10f, 3.0e-3f, 3.4e-7f}, {0.54f, 0.10f, 2.1e-5f, 1.4e-6f}}}};
+constexpr int kFormThreads = 1024;
+
+struct FormTime {
+  float lat, thr;  // us: the longest chain, all chains on one SM
+};
+__device__ __forceinline__ float form_cost(const float (&a)[4], const float (&f)[4]) {
+  return a[0] * f[0] + a[1] * f[1] + a[2] * f[2] + a[3] * f[3];
+}
+__global__ void __launch_bounds__(kFormThreads) pe_form_kernel(const BatchView B, FormCost one, FormCost team, int n_cap,
+                                                               float sms, int* counters) {
+  __shared__ FormTime part[2][kFormThreads / 32];
+  FormTime t[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+  for (int i = threadIdx.x; i < B.n_waveforms; i += kFormThreads) {
+    const float cap = (float)n_cap, lam = (float)B.lambda0[i];
+    const float s = (float)max(B.n_steps_arr ? B.n_steps_arr[i] : B.n_steps, 0);
+    const float n0 = B.z_init ? fminf(fmaxf((float)B.n_init[i], 0.0f), cap) : 0.0f;
+    const float goal = lam > 0.0f ? fminf(lam, cap) : 0.0f;  // (an invalid lambda0 runs no step)
+    const float ramp = fminf(s, fabsf(goal - n0) / kGrowth);
+    const float n1 = n0 + (goal > n0 ? kGrowth : -kGrowth) * ramp, flat = s - ramp;
+    // sums of N^0 .. N^3 over the steps
+    const float f[4] = {s, (n0 + n1) / 2 * ramp + n1 * flat, (n0 * n0 + n0 * n1 + n1 * n1) / 3 * ramp + n1 * n1 * flat,
+                        (n0 + n1) * (n0 * n0 + n1 * n1) / 4 * ramp + n1 * n1 * n1 * flat};
+    t[0].lat = fmaxf(t[0].lat, form_cost(one.lat, f));
+    t[1].lat = fmaxf(t[1].lat, form_cost(team.lat, f));
+    t[0].thr += form_cost(one.thr, f);
+    t[1].thr += form_cost(team.thr, f);
+  }
+  for (int k = 0; k < 2; ++k) {
+    for (int o = 16; o > 0; o >>= 1) {
+      t[k].lat = fmaxf(t[k].lat, __shfl_xor_sync(0xffffffffu, t[k].lat, o));
+      t[k].thr += __shfl_xor_sync(0xffffffffu, t[k].thr, o);
+    }
+    if ((threadIdx.x & 31) == 0) part[k][threadIdx.x / 32] = t[k];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float cube[2];
+    for (int k = 0; k < 2; ++k) {
+      float lat = 0.0f, thr = 0.0f;
+      for (int q = 0; q < kFormThreads / 32; ++q) {
+        lat = fmaxf(lat, part[k][q].lat);
+        thr += part[k][q].thr;
+      }
+      thr /= sms;
+      cube[k] = lat * lat * lat + thr * thr * thr;
+    }
+    const bool teams = cube[1] < cube[0];
+    counters[0] = teams ? B.n_waveforms : 0;
+    counters[1] = teams ? 0 : B.n_waveforms;
+    counters[2] = teams ? 1 : 0;
+  }
+}
+
+cudaError_t launch_pe_form(const DevModel& M, const BatchView& B, int sms, int* counters, cudaStream_t st) {
+  const FormCost(&c)[2] = kCost[pe_big(M.n_cap) ? 1 : 0];
+  pe_form_kernel<<<1, kFormThreads, 0, st>>>(B, c[0], c[1], M.n_cap, (float)sms, counters);
+  return cudaGetLastError();
+}
+
 // lambda_FSMP of given N histograms (testing aid): the device function every chain ends with,
 // one histogram per group of L lanes. Histogram i is h[i * (n_max + 1) .. (i + 1) * (n_max + 1)).
 template <int L>

@@ -2733,9 +2733,7 @@ cudaError_t pe_launch(const DevModel& M, const BatchView& B, int warps, int lane
   G.hist = hist;
   G.counter = counter;
   G.Ns = Ns;
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  e = with_pe_kernel<MIX>(M.precision, big, lanes, form, [&](auto k) {
+  const cudaError_t e = with_pe_kernel<MIX>(M.precision, big, lanes, form, [&](auto k) {
     k<<<ctas, warps * 32, smem, st>>>(M, B, G);
     return cudaSuccess;
   });

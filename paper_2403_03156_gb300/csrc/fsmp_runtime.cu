@@ -119,7 +119,7 @@ struct fsmp_ctx {
     void* cinv = nullptr;    // C^-1 slots
     double* ws = nullptr;    // FP64 refresh workspace slots
     int* hist = nullptr;     // N histogram slots
-    int* counter = nullptr;  // chain counter of the launch
+    int* counter = nullptr;  // chain counters of a launch in either form, and the form (launch_pe_form)
   };
   std::vector<PeSet> pe_sets;
   int pe_slots = 0, pe_warps = 4, pe_tile = 0, pe_lanes = 32;
@@ -130,7 +130,8 @@ struct fsmp_ctx {
   std::atomic<long long> n_launches{0};  // chain-kernel launches
   std::mutex tune_mu;                    // serialises fsmp_autotune calls
   std::mutex launch_mu;                  // the last PE-space launch (fsmp_last_launch)
-  fsmp_launch last_launch{};             // (lanes_per_chain 0: none yet)
+  fsmp_launch last_launch[2] = {};       // a warp per chain, a team (lanes_per_chain 0: not launched)
+  const int* last_form = nullptr;        // launched in both forms: the device's choice
   // serving loop
   std::vector<cudaStream_t> streams;
   cudaStream_t gmem_stream = nullptr;
@@ -312,55 +313,68 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
 }
 
 // Teams: a CTA of four warps per chain, which work together on what a chain of more than 32 PEs does
-// with C^-1. A chain is then about three times as fast, but an SM holds 4 of them instead of 8, and
-// chains of few PEs get nothing from it. So teams serve launches that end with their longest
-// chains: up to 20 chains per SM (mixture, 1000 steps: 3000 chains 16.7 ms against 17.5 with a warp
-// per chain, 4000 chains 22.9 against 20.2; uneven windows: 3000 chains 16.4 ms against 24.7, 6000
-// chains 32.9 against 30.1). A pile-up chain is beyond 32 PEs for all but its first steps: there
-// teams serve any number of chains that run for 512 steps or more (6000 chains x 1000 steps: 398 ms
-// against 643, x 600 steps 174 against 212, x 300 steps 60 against 47), or start from a given state,
-// and up to 8 chains per SM otherwise (1000 chains x 500 steps 23 ms against 30). Only where the
-// launch shape is left to the library, and where a chain can have clearly more than 32 PEs.
-constexpr int kTeamChains = 20, kTeamChainsBig = 8;  // most chains per SM
-constexpr int kTeamStepsBig = 512;
-constexpr int kTeamMinCap = 64;                      // least capacity
-bool pe_team_shape(const fsmp_ctx* c, const BatchView& B, PeShape* s) {
+// with C^-1. A chain is then two to three times as fast, but an SM holds 4 of them instead of 8 to 12
+// with a warp each. Where all chains of a launch are resident at once in teams, none waits for
+// another and a launch of light chains loses little (608 chains of lambda0 = 1: 5 %). Beyond, the
+// device compares the expected times of both forms (launch_pe_form), for up to 20 chains per SM (at
+// 30 a mix of 0.5 to 100 PEs is still 1.6 times as fast in teams, one of 0.5 to 50 as fast as
+// without) and for any number where a chain can be in pile-up (n_cap above 192: 6000 chains of 200
+// PEs x 600 steps 214 ms in teams, 228 without; of 5 PEs 22.7 and 14.0). Only where the launch shape
+// is left to the library, and where a chain can have clearly more than 32 PEs.
+constexpr int kTeamChains = 20;  // most chains per SM
+constexpr int kTeamMinCap = 64;  // least capacity
+enum TeamRule { kTeamNever, kTeamAlways, kTeamEstimate };
+TeamRule pe_team_rule(const fsmp_ctx* c, const BatchView& B, PeShape* s) {
   const bool big = pe_big(c->p.n_cap);
   if (c->p.threads_per_chain != 0 || c->p.pe_ctas_per_sm != 0 || c->p.n_cap < kTeamMinCap ||
       !pe_team_ok(c->p.precision, c->pe_lanes))
-    return false;
-  const bool few = B.n_waveforms <= (big ? kTeamChainsBig : kTeamChains) * c->prop.multiProcessorCount;
-  const bool long_big = big && (B.z_init || (!B.n_steps_arr && B.n_steps >= kTeamStepsBig));
-  if (!c->pe_team_always && !(c->pe_tile_free && (few || long_big))) return false;
+    return kTeamNever;
+  const bool in_range = big || B.n_waveforms <= kTeamChains * c->prop.multiProcessorCount;
+  if (!c->pe_team_always && !(c->pe_tile_free && in_range)) return kTeamNever;
   PeShape t;
   t.form = kPeTeam;
   t.warps = 4;
   t.tile = c->pe_tile;  // 40; 96: a burst of 64 events 57 ms against 51, pile-up 245 against 255
   t.smem = pe_smem_bytes(c->M, B.n_max, t.warps, c->pe_lanes, t.tile, t.form);
-  if (t.smem > (size_t)c->prop.sharedMemPerBlockOptin) return false;
+  if (t.smem > (size_t)c->prop.sharedMemPerBlockOptin) return kTeamNever;
   const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, c->pe_lanes, c->M.n_comp > 1, t.form);
-  if (per_sm < 1) return false;
-  t.ctas = per_sm * c->prop.multiProcessorCount;
+  if (per_sm < 1) return kTeamNever;
+  t.ctas = std::min(per_sm * c->prop.multiProcessorCount, c->pe_slots);
   *s = t;
-  return true;
+  return c->pe_team_always || B.n_waveforms <= t.ctas ? kTeamAlways : kTeamEstimate;
 }
 
 int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   if (c->pe_sets.empty()) FAIL(FSMP_ERR_INVALID, "the PE-space kernel was not set up at fsmp_create");
   if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
-  PeShape s;
+  PeShape s, t;
   if (pe_shape(c, B.n_max, B.n_waveforms, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
-  pe_team_shape(c, B, &s);
-  const bool team = s.form == kPeTeam;
-  const int cpc = team ? 1 : s.warps * (32 / c->pe_lanes);
-  const int ctas = std::min(std::min(s.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
+  const TeamRule rule = pe_team_rule(c, B, &t);
   const fsmp_ctx::PeSet& ps = c->pe_sets[set];
-  cudaError_t e = launch_pe(c->M, B, s.warps, c->pe_lanes, ctas, s.tile, s.smem, ps.cinv, c->pe_c_stride,
-                            ps.ws, c->pe_ws_stride, ps.hist, ps.counter, s.form, st);
+  fsmp_launch made[2] = {};
+  auto launch = [&](const PeShape& f, int* counter) {
+    const bool team = f.form == kPeTeam;
+    const int cpc = team ? 1 : f.warps * (32 / c->pe_lanes);
+    const int ctas = std::min(std::min(f.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
+    made[team] = fsmp_launch{c->pe_lanes, cpc, f.tile, ctas, team ? 1 : 0};
+    return launch_pe(c->M, B, f.warps, c->pe_lanes, ctas, f.tile, f.smem, ps.cinv, c->pe_c_stride, ps.ws,
+                     c->pe_ws_stride, ps.hist, counter, f.form, st);
+  };
+  cudaError_t e;
+  if (rule == kTeamEstimate) {  // the two launches share the slots: one follows the other, and runs no chain
+    e = launch_pe_form(c->M, B, c->prop.multiProcessorCount, ps.counter, st);
+    if (e == cudaSuccess) e = launch(t, ps.counter + 1);
+    if (e == cudaSuccess) e = launch(s, ps.counter);
+  } else {
+    e = cudaMemsetAsync(ps.counter, 0, sizeof(int), st);
+    if (e == cudaSuccess) e = launch(rule == kTeamAlways ? t : s, ps.counter);
+  }
   c->n_launches++;
   if (e != cudaSuccess) { set_error("launch_pe", cudaGetErrorString(e), __LINE__); return FSMP_ERR_CUDA; }
   std::lock_guard<std::mutex> lk(c->launch_mu);
-  c->last_launch = fsmp_launch{c->pe_lanes, cpc, s.tile, ctas, team ? 1 : 0};
+  c->last_launch[0] = made[0];
+  c->last_launch[1] = made[1];
+  c->last_form = rule == kTeamEstimate ? ps.counter + 2 : nullptr;
   return FSMP_OK;
 }
 
@@ -1014,8 +1028,8 @@ int fsmp_create(const fsmp_params* params, fsmp_ctx** out) {
       if (cb && cudaMalloc(&ps.cinv, cb) != cudaSuccess) FAIL(FSMP_ERR_NOMEM, "PE-space C^-1 slots");
       if (wb && cudaMalloc((void**)&ps.ws, wb) != cudaSuccess) FAIL(FSMP_ERR_NOMEM, "PE-space refresh workspace");
       if (cudaMalloc((void**)&ps.hist, hb) != cudaSuccess) FAIL(FSMP_ERR_NOMEM, "PE-space N histograms");
-      CK(cudaMalloc((void**)&ps.counter, sizeof(int)));
-      c->pe_bytes += cb + wb + hb + sizeof(int);
+      CK(cudaMalloc((void**)&ps.counter, 3 * sizeof(int)));
+      c->pe_bytes += cb + wb + hb + 3 * sizeof(int);
       c->pe_sets.push_back(ps);
     }
   }
@@ -1297,8 +1311,10 @@ int fsmp_last_launch(fsmp_ctx* c, fsmp_launch* out) {
   g_last_error[0] = 0;
   if (!c || !out) return FSMP_ERR_INVALID;
   std::lock_guard<std::mutex> lk(c->launch_mu);
-  if (c->last_launch.lanes_per_chain == 0) FAIL(FSMP_ERR_INVALID, "the context has made no PE-space launch");
-  *out = c->last_launch;
+  int team = c->last_launch[1].lanes_per_chain != 0;
+  if (!team && c->last_launch[0].lanes_per_chain == 0) FAIL(FSMP_ERR_INVALID, "the context has made no PE-space launch");
+  if (c->last_form) CK(cudaMemcpy(&team, c->last_form, sizeof(int), cudaMemcpyDeviceToHost));
+  *out = c->last_launch[team];
   return FSMP_OK;
 }
 

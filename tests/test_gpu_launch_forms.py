@@ -85,3 +85,46 @@ def test_no_launch_yet():
         with pytest.raises(fsmp.FsmpError) as e:
             ctx.last_launch()
     assert e.value.code == fsmp.ERR_INVALID
+
+
+@pytest.mark.parametrize("workload,n_cap,lam,steps,team", [
+    ("batched_uneven_100k", 128, (8.0, 8.0), 200, 0),     # light: a warp per chain
+    ("batched_uneven_100k", 128, (0.2, 2.0), 200, 0),
+    ("batched_uneven_100k", 64, (0.2, 2.0), 200, 0),
+    ("batched_uneven_100k", 128, (0.5, 100.0), 400, 1),   # a tail of heavy chains: teams
+    ("mcp_uneven_20k", 128, (5.0, 15.0), 200, 0),
+    ("mcp_uneven_20k", 128, (0.5, 100.0), 400, 1),
+    ("highpileup_20k_1024", 384, (0.5, 5.0), 200, 0),
+    ("highpileup_20k_1024", 384, (100.0, 200.0), 600, 1)])
+def test_the_form_follows_the_chains(workload, n_cap, lam, steps, team):
+    """1300 chains, more than the GPU holds as teams: the form follows their lambda0 and steps, on the
+    device-resident path and from host memory alike; a lambda0 that is not a number spoils its own
+    chain only; and the outputs are those of one warp per chain."""
+    pytest.importorskip("torch")
+    W = 1300
+    p = dict(workloads.CONFIGS[workload]["params"], n_cap=n_cap, precision=fsmp.FP32_REFRESH, refresh_every=16, pe_lanes=32,
+             n_max=1024, n_streams=1)
+    b = _simulate(workload, np.geomspace(lam[1], lam[0], W))
+    b["lambda0"][7] = np.nan
+    got, launch = _run(p, b, steps)
+    ref, _ = _run(dict(p, **ONE_WARP), b, steps)
+    assert launch["team"] == team and launch["chains_per_cta"] == (1 if team else 4)
+    assert np.array_equal(np.nonzero(got[0].view(fsmp.SUMMARY_DTYPE)["status"] & fsmp.ST_INVALID)[0], [7])
+    for a, c in zip(got, ref):
+        np.testing.assert_array_equal(a, c)
+    host = dict(b, lambda0=np.where(np.isnan(b["lambda0"]), lam[0], b["lambda0"]), n_steps=steps, burn_in=10, seed=9, index_base=0)
+    for k in ("T_lo", "T_hi", "wf_ids"):
+        host.pop(k, None)
+    with gpu_util.context(p) as ctx:
+        s, _ = ctx.run(host)
+        assert ctx.last_launch()["team"] == team
+    others = np.arange(W) != 7
+    assert s[others].tobytes() == got[0].view(fsmp.SUMMARY_DTYPE)[others].tobytes()
+
+
+def test_short_chains_take_no_team():
+    """A chain of 100 steps does not get far beyond 20 PEs, whatever its lambda0."""
+    pytest.importorskip("torch")
+    for workload, n_cap in (("batched_uneven_100k", 128), ("highpileup_20k_1024", 384)):
+        p = dict(workloads.CONFIGS[workload]["params"], n_cap=n_cap, precision=fsmp.FP32_REFRESH, n_max=1024, n_streams=1)
+        assert _run(p, _simulate(workload, np.full(1300, 60.0)), 100)[1]["team"] == 0
