@@ -126,6 +126,7 @@ struct fsmp_ctx {
   bool pe_lanes_free = false;  // pe_lanes left to fsmp_autotune
   bool pe_team_always = false;  // fsmp_autotune found teams faster on its batch
   bool pe_tile_free = false;   // pe_tile neither given nor tuned
+  int pe_limit_warps = 4, pe_limit_tile = 0, pe_limit_lanes = 32;  // the created shape, for pe_limit_bytes
   size_t pe_c_stride = 0, pe_ws_stride = 0, pe_bytes = 0;
   std::atomic<long long> n_launches{0};  // chain-kernel launches
   std::mutex tune_mu;                    // serialises fsmp_autotune calls
@@ -277,8 +278,9 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
   const bool many = n_chains > kMoreChains * c->prop.multiProcessorCount || c->p.n_cap < kMoreCap;
   const bool more = pe_more_ok(c->M, c->pe_lanes) && (c->p.pe_ctas_per_sm > 0 ? c->p.pe_ctas_per_sm > 2 : many);
   s->form = more ? kPeWarpMore : kPeWarp;
-  const int tile = c->pe_tile_free ? std::min(c->p.n_cap, 32) : c->pe_tile;
-  if (pe_limit_bytes(c->M, n_alloc, c->pe_warps, c->pe_lanes, tile) > (size_t)c->prop.sharedMemPerBlockOptin)
+  // the limit is the created context's, whatever shape was tuned
+  if (pe_limit_bytes(c->M, n_alloc, c->pe_limit_warps, c->pe_limit_lanes, c->pe_limit_tile) >
+      (size_t)c->prop.sharedMemPerBlockOptin)
     return FSMP_ERR_INVALID;
   s->warps = c->pe_warps;
   s->tile = c->pe_tile;
@@ -1003,6 +1005,9 @@ int fsmp_create(const fsmp_params* params, fsmp_ctx** out) {
     c->pe_lanes = p.pe_lanes > 0 ? p.pe_lanes : 32;
     c->pe_lanes_free = p.pe_lanes == 0 && pe_lanes_ok(16, p.n_cap);
     c->pe_tile_free = p.pe_tile == 0;
+    c->pe_limit_warps = c->pe_warps;
+    c->pe_limit_tile = c->pe_tile_free ? std::min(p.n_cap, kTileSmall) : c->pe_tile;
+    c->pe_limit_lanes = c->pe_lanes;
     c->pe_c_stride = c->pe_tile < p.n_cap ? pe_c_entries(p.n_cap) : 0;
     CK(pe_kernel_attributes(p.precision, max_smem));
     int slots = 0;
