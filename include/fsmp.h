@@ -325,14 +325,15 @@ int fsmp_gelman_rubin(const fsmp_summary* chains, int m, int field, double* rhat
 int fsmp_gelman_diag(const fsmp_summary* chains, int m, int field, double confidence, double* rhat,
                      double* upper);
 
-/* Launch shape of the PE-space kernel chosen by fsmp_autotune. */
+/* What fsmp_autotune reports: the launch that the tuned batch will be (for a team per chain, see
+ * fsmp_launch, chains_per_cta is 1 and ctas_per_sm 0). */
 typedef struct {
   int pe_tile;                   /* PEs per chain whose C^-1 stays in shared memory          */
   int chains_per_cta;            /* chains per CTA (warps x 32 / lanes_per_chain)            */
   int ctas_per_sm;               /* resident CTAs per SM (0: as many as fit)                 */
-  int n_tried;                   /* candidate shapes timed                                   */
-  double best_steps_per_s;       /* MCMC steps/s of the chosen shape on the trial            */
-  double default_steps_per_s;    /* the same for the shape the context started with          */
+  int n_tried;                   /* launches timed                                           */
+  double best_steps_per_s;       /* MCMC steps/s of that launch on the trial                 */
+  double default_steps_per_s;    /* the same for the launch before tuning                    */
   int lanes_per_chain;           /* 32 or 16                                                  */
 } fsmp_tune;
 
@@ -340,9 +341,15 @@ typedef struct {
  * batch laid out as for fsmp_run_device: time trial runs of its first `sample` waveforms for
  * `trial_steps` MCMC steps in each candidate shape -- lanes per chain (only if the context
  * was created with pe_lanes = 0), shared-memory tile of C^-1, warps per CTA and resident CTAs
- * per SM, and a CTA of four warps per chain -- and keep the fastest for the context's later launches. The batch's own output and
+ * per SM -- and keep the fastest for the context's later launches. A candidate has to be 1 %
+ * faster than the shape it replaces. Whether a launch gives each chain a team of four warps
+ * instead stays a matter of that launch's own chains: the batch, lambda0 and n_steps (trial_steps
+ * if 0) here say whether the tuned batch will be one, and 16 lanes, which run no teams, are taken
+ * only where they are faster than that. A team is timed for batches of more chains than the
+ * library gives teams to; where it is faster, later launches of any size may take teams. Choose
+ * `sample` large enough to fill the GPU if the batch does. The batch's own output and
  * trace buffers are not touched (the trials write to scratch). Later results do not depend on
- * the tile, warps or CTAs: a chain's arithmetic is the same in each. They do depend, up to
+ * the tile, warps, CTAs or teams: a chain's arithmetic is the same in each. They do depend, up to
  * rounding, on the lane count; fix pe_lanes for results reproducible bit for bit.
  * Blocks until the trials finish. Call it with no request in flight on the context. Returns
  * FSMP_OK (out, if not NULL, describes the choice), FSMP_ERR_INVALID (not a PE-space context,

@@ -122,11 +122,15 @@ struct fsmp_ctx {
     int* counter = nullptr;  // chain counters of a launch in either form, and the form (launch_pe_form)
   };
   std::vector<PeSet> pe_sets;
-  int pe_slots = 0, pe_warps = 4, pe_tile = 0, pe_lanes = 32;
+  // How chains are launched, as created (pe0) and as fsmp_autotune left it (pe; under launch_mu)
+  struct PeConfig {
+    int warps = 4, tile = 0, lanes = 32;
+    int ctas = 0;           // resident CTAs per SM (0: as many as fit)
+    bool tile_free = false;  // the tile neither given nor tuned
+    bool team_any = false;   // the estimate may choose teams for any number of chains
+  } pe, pe0;
+  int pe_slots = 0;
   bool pe_lanes_free = false;  // pe_lanes left to fsmp_autotune
-  bool pe_team_always = false;  // fsmp_autotune found teams faster on its batch
-  bool pe_tile_free = false;   // pe_tile neither given nor tuned
-  int pe_limit_warps = 4, pe_limit_tile = 0, pe_limit_lanes = 32;  // the created shape, for pe_limit_bytes
   size_t pe_c_stride = 0, pe_ws_stride = 0, pe_bytes = 0;
   std::atomic<long long> n_launches{0};  // chain-kernel launches
   std::mutex tune_mu;                    // serialises fsmp_autotune calls
@@ -274,18 +278,18 @@ struct PeShape {
 // of 2 to 32 PEs are 0 to 24 % faster in it, of 0.5 to 50 PEs 15 to 30 % slower.)
 constexpr int kMoreChains = 40;  // chains per SM
 constexpr int kMoreCap = 64;     // n_cap below
-int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
+int pe_shape(const fsmp_ctx* c, const fsmp_ctx::PeConfig& g, int n_alloc, int n_chains, PeShape* s) {
   const bool many = n_chains > kMoreChains * c->prop.multiProcessorCount || c->p.n_cap < kMoreCap;
-  const bool more = pe_more_ok(c->M, c->pe_lanes) && (c->p.pe_ctas_per_sm > 0 ? c->p.pe_ctas_per_sm > 2 : many);
+  const bool more = pe_more_ok(c->M, g.lanes) && (g.ctas > 0 ? g.ctas > 2 : many);
   s->form = more ? kPeWarpMore : kPeWarp;
   // the limit is the created context's, whatever shape was tuned
-  if (pe_limit_bytes(c->M, n_alloc, c->pe_limit_warps, c->pe_limit_lanes, c->pe_limit_tile) >
-      (size_t)c->prop.sharedMemPerBlockOptin)
+  const int tile = c->pe0.tile_free ? std::min(c->p.n_cap, kTileSmall) : c->pe0.tile;
+  if (pe_limit_bytes(c->M, n_alloc, c->pe0.warps, c->pe0.lanes, tile) > (size_t)c->prop.sharedMemPerBlockOptin)
     return FSMP_ERR_INVALID;
-  s->warps = c->pe_warps;
-  s->tile = c->pe_tile;
+  s->warps = g.warps;
+  s->tile = g.tile;
   for (;;) {
-    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, s->tile, s->form);
+    s->smem = pe_smem_bytes(c->M, n_alloc, s->warps, g.lanes, s->tile, s->form);
     if (s->smem <= (size_t)c->prop.sharedMemPerBlockOptin) break;
     const bool slots = c->pe_c_stride > 0;  // room for C^-1 beyond the tile
     if (slots && s->tile > 16) s->tile = std::max(16, s->tile - 8);
@@ -294,7 +298,7 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
     else return FSMP_ERR_INVALID;
   }
   auto occupancy = [&](size_t smem) {
-    return pe_kernel_occupancy(c->p.precision, s->warps * 32, smem, pe_big(c->p.n_cap), c->pe_lanes, c->M.n_comp > 1,
+    return pe_kernel_occupancy(c->p.precision, s->warps * 32, smem, pe_big(c->p.n_cap), g.lanes, c->M.n_comp > 1,
                                s->form);
   };
   int per_sm = occupancy(s->smem);
@@ -303,13 +307,13 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
   // KB more per CTA kept half of the chains out (pile-up model of 1024 samples, 2 CTAs per SM instead
   // of 1: 6000 chains of 2 PEs x 300 steps 6.4 ms against 9.1, of 35 PEs 32.0 and 31.0; FP64, n_cap
   // 128, windows of 400: 2000 chains of 15 PEs x 60 steps 4.8 and 5.2).
-  const int resident = per_sm * c->prop.multiProcessorCount * s->warps * (32 / c->pe_lanes);
-  if (c->pe_tile_free && c->pe_c_stride > 0 && s->tile > kTileSmall && n_chains > resident) {
-    const size_t smem = pe_smem_bytes(c->M, n_alloc, s->warps, c->pe_lanes, kTileSmall, s->form);
-    const int more = occupancy(smem);
-    if (more > per_sm) { per_sm = more; s->tile = kTileSmall; s->smem = smem; }
+  const int resident = per_sm * c->prop.multiProcessorCount * s->warps * (32 / g.lanes);
+  if (g.tile_free && c->pe_c_stride > 0 && s->tile > kTileSmall && n_chains > resident) {
+    const size_t smem = pe_smem_bytes(c->M, n_alloc, s->warps, g.lanes, kTileSmall, s->form);
+    const int more_ctas = occupancy(smem);
+    if (more_ctas > per_sm) { per_sm = more_ctas; s->tile = kTileSmall; s->smem = smem; }
   }
-  if (c->p.pe_ctas_per_sm > 0) per_sm = std::min(per_sm, c->p.pe_ctas_per_sm);
+  if (g.ctas > 0) per_sm = std::min(per_sm, g.ctas);
   s->ctas = per_sm * c->prop.multiProcessorCount;
   return FSMP_OK;
 }
@@ -321,45 +325,45 @@ int pe_shape(const fsmp_ctx* c, int n_alloc, int n_chains, PeShape* s) {
 // device compares the expected times of both forms (launch_pe_form), for up to 20 chains per SM (at
 // 30 a mix of 0.5 to 100 PEs is still 1.6 times as fast in teams, one of 0.5 to 50 as fast as
 // without) and for any number where a chain can be in pile-up (n_cap above 192: 6000 chains of 200
-// PEs x 600 steps 214 ms in teams, 228 without; of 5 PEs 22.7 and 14.0). Only where the launch shape
-// is left to the library, and where a chain can have clearly more than 32 PEs.
+// PEs x 600 steps 214 ms in teams, 228 without; of 5 PEs 22.7 and 14.0), or where fsmp_autotune timed
+// teams as the faster form. Only where the launch shape is left to the library, and where a chain can
+// have clearly more than 32 PEs. A shape that fsmp_autotune chose is the one-warp form's, and leaves
+// the rule as it is.
 constexpr int kTeamChains = 20;  // most chains per SM
 constexpr int kTeamMinCap = 64;  // least capacity
 enum TeamRule { kTeamNever, kTeamAlways, kTeamEstimate };
-TeamRule pe_team_rule(const fsmp_ctx* c, const BatchView& B, PeShape* s) {
+TeamRule pe_team_rule(const fsmp_ctx* c, const fsmp_ctx::PeConfig& g, const BatchView& B, PeShape* s) {
   const bool big = pe_big(c->p.n_cap);
   if (c->p.threads_per_chain != 0 || c->p.pe_ctas_per_sm != 0 || c->p.n_cap < kTeamMinCap ||
-      !pe_team_ok(c->p.precision, c->pe_lanes))
+      !pe_team_ok(c->p.precision, g.lanes))
     return kTeamNever;
   const bool in_range = big || B.n_waveforms <= kTeamChains * c->prop.multiProcessorCount;
-  if (!c->pe_team_always && !(c->pe_tile_free && in_range)) return kTeamNever;
+  if (!g.team_any && !(c->pe0.tile_free && in_range)) return kTeamNever;
   PeShape t;
   t.form = kPeTeam;
   t.warps = 4;
-  t.tile = c->pe_tile;  // 40; 96: a burst of 64 events 57 ms against 51, pile-up 245 against 255
-  t.smem = pe_smem_bytes(c->M, B.n_max, t.warps, c->pe_lanes, t.tile, t.form);
+  t.tile = c->pe0.tile;  // 40; 96: a burst of 64 events 57 ms against 51, pile-up 245 against 255
+  t.smem = pe_smem_bytes(c->M, B.n_max, t.warps, g.lanes, t.tile, t.form);
   if (t.smem > (size_t)c->prop.sharedMemPerBlockOptin) return kTeamNever;
-  const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, c->pe_lanes, c->M.n_comp > 1, t.form);
+  const int per_sm = pe_kernel_occupancy(c->p.precision, t.warps * 32, t.smem, big, g.lanes, c->M.n_comp > 1, t.form);
   if (per_sm < 1) return kTeamNever;
   t.ctas = std::min(per_sm * c->prop.multiProcessorCount, c->pe_slots);
   *s = t;
-  return c->pe_team_always || B.n_waveforms <= t.ctas ? kTeamAlways : kTeamEstimate;
+  return B.n_waveforms <= t.ctas ? kTeamAlways : kTeamEstimate;
 }
 
-int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
-  if (c->pe_sets.empty()) FAIL(FSMP_ERR_INVALID, "the PE-space kernel was not set up at fsmp_create");
-  if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
-  PeShape s, t;
-  if (pe_shape(c, B.n_max, B.n_waveforms, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
-  const TeamRule rule = pe_team_rule(c, B, &t);
+// Launch the chains of B in the slots of `set`: a warp per chain in shape s, or a team in shape t,
+// or whichever the device's estimate chooses.
+int launch_chains(fsmp_ctx* c, const BatchView& B, int set, TeamRule rule, const PeShape& s, const PeShape& t, int lanes,
+                  cudaStream_t st) {
   const fsmp_ctx::PeSet& ps = c->pe_sets[set];
   fsmp_launch made[2] = {};
   auto launch = [&](const PeShape& f, int* counter) {
     const bool team = f.form == kPeTeam;
-    const int cpc = team ? 1 : f.warps * (32 / c->pe_lanes);
+    const int cpc = team ? 1 : f.warps * (32 / lanes);
     const int ctas = std::min(std::min(f.ctas, c->pe_slots / cpc), (B.n_waveforms + cpc - 1) / cpc);
-    made[team] = fsmp_launch{c->pe_lanes, cpc, f.tile, ctas, team ? 1 : 0};
-    return launch_pe(c->M, B, f.warps, c->pe_lanes, ctas, f.tile, f.smem, ps.cinv, c->pe_c_stride, ps.ws,
+    made[team] = fsmp_launch{lanes, cpc, f.tile, ctas, team ? 1 : 0};
+    return launch_pe(c->M, B, f.warps, lanes, ctas, f.tile, f.smem, ps.cinv, c->pe_c_stride, ps.ws,
                      c->pe_ws_stride, ps.hist, counter, f.form, st);
   };
   cudaError_t e;
@@ -378,6 +382,21 @@ int run_pe(fsmp_ctx* c, BatchView B, int set, cudaStream_t st) {
   c->last_launch[1] = made[1];
   c->last_form = rule == kTeamEstimate ? ps.counter + 2 : nullptr;
   return FSMP_OK;
+}
+
+fsmp_ctx::PeConfig pe_config(fsmp_ctx* c) {
+  std::lock_guard<std::mutex> lk(c->launch_mu);
+  return c->pe;
+}
+
+int run_pe(fsmp_ctx* c, const BatchView& B, int set, cudaStream_t st) {
+  if (c->pe_sets.empty()) FAIL(FSMP_ERR_INVALID, "the PE-space kernel was not set up at fsmp_create");
+  if (B.n_max > c->p.n_max) FAIL(FSMP_ERR_INVALID, "window longer than n_max");
+  const fsmp_ctx::PeConfig g = pe_config(c);
+  PeShape s, t;
+  if (pe_shape(c, g, B.n_max, B.n_waveforms, &s) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
+  const TeamRule rule = pe_team_rule(c, g, B, &t);
+  return launch_chains(c, B, set, rule, s, t, g.lanes, st);
 }
 
 int run_view(fsmp_ctx* c, BatchView B, cudaStream_t st, int set) {
@@ -997,30 +1016,29 @@ int fsmp_create(const fsmp_params* params, fsmp_ctx** out) {
   // refresh workspace (FP32 mode) and of the N histogram, one set per launch stream; enough
   // slots for every shape the context may launch (both lane counts when the tuner picks it)
   if (p.kernel == FSMP_KERNEL_PE) {
-    c->pe_warps = p.threads_per_chain > 0 ? std::min(4, p.threads_per_chain / 32) : 4;
+    fsmp_ctx::PeConfig& g = c->pe0;
+    g.warps = p.threads_per_chain > 0 ? std::min(4, p.threads_per_chain / 32) : 4;
     const size_t esz = pe_c_entry_bytes(p.precision);
     // default tile: 40 PEs leaves the L1 the global slots are read through its size (pile-up, 600
     // chains: 85.6 ms, 89.4 with 48 and 94.7 with 32; the same for the serving model, n_cap 192)
-    c->pe_tile = p.pe_tile > 0 ? std::min(p.pe_tile, p.n_cap) : std::min(p.n_cap, 40);
-    c->pe_lanes = p.pe_lanes > 0 ? p.pe_lanes : 32;
+    g.tile = p.pe_tile > 0 ? std::min(p.pe_tile, p.n_cap) : std::min(p.n_cap, 40);
+    g.lanes = p.pe_lanes > 0 ? p.pe_lanes : 32;
+    g.ctas = p.pe_ctas_per_sm;
+    g.tile_free = p.pe_tile == 0;
+    c->pe = g;
     c->pe_lanes_free = p.pe_lanes == 0 && pe_lanes_ok(16, p.n_cap);
-    c->pe_tile_free = p.pe_tile == 0;
-    c->pe_limit_warps = c->pe_warps;
-    c->pe_limit_tile = c->pe_tile_free ? std::min(p.n_cap, kTileSmall) : c->pe_tile;
-    c->pe_limit_lanes = c->pe_lanes;
-    c->pe_c_stride = c->pe_tile < p.n_cap ? pe_c_entries(p.n_cap) : 0;
+    c->pe_c_stride = g.tile < p.n_cap ? pe_c_entries(p.n_cap) : 0;
     CK(pe_kernel_attributes(p.precision, max_smem));
     int slots = 0;
-    const int lanes0 = c->pe_lanes;
     for (int lanes : {32, 16}) {
-      if (lanes != lanes0 && !c->pe_lanes_free) continue;
-      c->pe_lanes = lanes;
+      if (lanes != g.lanes && !c->pe_lanes_free) continue;
+      fsmp_ctx::PeConfig l = g;
+      l.lanes = lanes;
       for (int nn : {std::min(64, p.n_max), p.n_max}) {
         PeShape s;
-        if (pe_shape(c.get(), nn, INT_MAX, &s) == FSMP_OK) slots = std::max(slots, s.ctas * s.warps * (32 / lanes));
+        if (pe_shape(c.get(), l, nn, INT_MAX, &s) == FSMP_OK) slots = std::max(slots, s.ctas * s.warps * (32 / lanes));
       }
     }
-    c->pe_lanes = lanes0;
     if (slots < 1) FAIL(FSMP_ERR_INVALID, "n_max too large for the PE-space kernel");
     c->pe_slots = slots;
     // the FP64 rebuild runs in FP32 mode every K accepts, and in both modes for a chain that
@@ -1188,6 +1206,15 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   B.index_base = b->index_base;
   B.samples = b->samples; B.offsets = b->offsets; B.lambda0 = b->lambda0; B.t_origin = b->t_origin_ns;
   B.T_lo = b->T_lo; B.T_hi = b->T_hi; B.t0_init = b->t0_init; B.wf_ids = b->wf_ids;
+  // the batch as it will be launched, for the rule on teams
+  BatchView full = B;
+  full.n_waveforms = b->n_waveforms;
+  if (b->n_steps > 0) full.n_steps = b->n_steps;
+  if (b->z_init && b->n_init) { full.z_init = b->z_init; full.n_init = b->n_init; full.z_stride = b->z_stride; }
+  const fsmp_ctx::PeConfig base = pe_config(c);
+  fsmp_ctx::PeConfig best_g = base;
+  PeShape warp0, team{};
+  if (pe_shape(c, base, B.n_max, b->n_waveforms, &warp0) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
   fsmp_summary* scratch = nullptr;
   CK(cudaMalloc(&scratch, sizeof(fsmp_summary) * (size_t)W));
   B.out = scratch;
@@ -1197,19 +1224,12 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   const int set = (int)c->streams.size();
-  const int tile0 = c->pe_tile, warps0 = c->pe_warps, ctas0 = c->p.pe_ctas_per_sm, lanes0 = c->pe_lanes;
-  const bool tfree0 = c->pe_tile_free;
-  const bool team0 = c->pe_team_always;
-  c->pe_team_always = false;
-  auto trial = [&](int lanes, int tile, int warps, int ctas, double* rate) -> int {
-    c->pe_lanes = lanes; c->pe_tile = tile; c->pe_warps = warps; c->p.pe_ctas_per_sm = ctas;
-    PeShape s;
-    // (the default shape, timed first, is taken as pe_shape makes it)
-    if (pe_shape(c, B.n_max, B.n_waveforms, &s) != FSMP_OK || (!c->pe_tile_free && (s.warps != warps || s.tile != tile))) { *rate = -1.0; return FSMP_OK; }
+  int n_tried = 0;
+  auto timed = [&](TeamRule rule, const PeShape& s, int lanes, double* rate) -> int {
     float best_ms = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {  // the first run warms the caches and the code
       if (cudaEventRecord(e0, st) != cudaSuccess) return FSMP_ERR_CUDA;
-      int rc = run_pe(c, B, set, st);
+      int rc = launch_chains(c, B, set, rule, s, team, lanes, st);
       if (rc) return rc;
       if (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) return FSMP_ERR_CUDA;
       float ms = 0.f;
@@ -1217,6 +1237,29 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
       if (rep > 0) best_ms = std::min(best_ms, ms);
     }
     *rate = (double)W * trial_steps / (best_ms * 1e-3);
+    ++n_tried;
+    return FSMP_OK;
+  };
+  // a warp per chain in the shape that g names (not one that had to be made smaller to fit)
+  auto trial = [&](fsmp_ctx::PeConfig g, double* rate) -> int {
+    PeShape s;
+    g.tile_free = false;
+    *rate = -1.0;
+    if (pe_shape(c, g, B.n_max, b->n_waveforms, &s) != FSMP_OK || s.warps != g.warps || s.tile != g.tile) return FSMP_OK;
+    return timed(kTeamNever, s, g.lanes, rate);
+  };
+  // whether a launch of the whole batch is one in teams (then in shape `team`)
+  auto in_teams = [&](const fsmp_ctx::PeConfig& g, bool* yes) -> int {
+    const TeamRule rule = pe_team_rule(c, g, full, &team);
+    int v = rule == kTeamAlways;
+    if (rule == kTeamEstimate) {
+      int* const counter = c->pe_sets[set].counter;
+      if (launch_pe_form(c->M, full, c->prop.multiProcessorCount, counter, st) != cudaSuccess ||
+          cudaMemcpyAsync(&v, counter + 2, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+          cudaStreamSynchronize(st) != cudaSuccess)
+        return FSMP_ERR_CUDA;
+    }
+    *yes = v != 0;
     return FSMP_OK;
   };
   // candidates: a tile needs the global C^-1 slots unless it covers n_cap
@@ -1224,73 +1267,85 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   std::vector<int> tiles;
   for (int t : {8, 16, 24, 32, 48, 64})
     if (t < c->p.n_cap ? have_slots : true) tiles.push_back(std::min(t, c->p.n_cap));
-  if (!have_slots) tiles = {tile0};
+  if (!have_slots) tiles = {base.tile};
   std::sort(tiles.begin(), tiles.end());
   tiles.erase(std::unique(tiles.begin(), tiles.end()), tiles.end());
-  double r0 = 0.0, best = -1.0;
-  int bl = lanes0, bt = tile0, bw = warps0, bc = ctas0, n_tried = 0;
-  bool bteam = false;
-  int rc = trial(lanes0, tile0, warps0, ctas0, &r0);  // the default launch, a team per chain where its rule says so
-  c->pe_tile_free = false;  // the other trials run in the shapes they name, later launches in the chosen one
-  if (rc == FSMP_OK) {
-    best = r0; ++n_tried;
-    // coordinate search: lanes per chain (when the context leaves it free), tile, warps per
-    // CTA, then resident CTAs per SM
-    if (c->pe_lanes_free) {
-      for (int l : {32, 16}) {
-        double r;
-        if (l == lanes0) continue;
-        if ((rc = trial(l, bt, bw, bc, &r)) != FSMP_OK) break;
-        ++n_tried;
-        if (r > best) { best = r; bl = l; }
-      }
+  // What is tuned is the shape of a launch with a warp per chain; launches in teams keep their rule,
+  // which looks at each launch's own chains. A candidate has to be more than 1 % faster (runs of one
+  // shape differ by that).
+  constexpr double kFaster = 1.01;
+  double r0 = 0.0, best = -1.0, r_team = -1.0, r = -1.0;
+  bool teams = false;
+  int rc = timed(kTeamNever, warp0, base.lanes, &r0);  // the launch as the context makes it now
+  best = r0;
+  if (rc == FSMP_OK) rc = in_teams(base, &teams);
+  if (rc == FSMP_OK && teams) rc = timed(kTeamAlways, warp0, base.lanes, &r_team);
+  const double r_default = teams ? r_team : r0;
+  auto consider = [&](const fsmp_ctx::PeConfig& g, double than) {
+    if (rc != FSMP_OK || (rc = trial(g, &r)) != FSMP_OK || r <= than * kFaster) return;
+    best = r;
+    best_g = g;
+    best_g.tile_free = false;
+  };
+  // coordinate search: lanes per chain (when the context leaves it free; 16 lanes run no teams, so
+  // they have to beat those too), tile, warps per CTA, then resident CTAs per SM
+  if (c->pe_lanes_free)
+    for (int l : {32, 16}) {
+      fsmp_ctx::PeConfig g = best_g;
+      g.lanes = l;
+      if (l != base.lanes) consider(g, std::max(best, r_team));
     }
-    for (int t : tiles) {
-      double r;
-      if (rc != FSMP_OK || (rc = trial(bl, t, bw, bc, &r)) != FSMP_OK) break;
-      ++n_tried;
-      if (r > best) { best = r; bt = t; }
-    }
-    for (int w : {1, 2, 4}) {
-      double r;
-      if (rc != FSMP_OK || (rc = trial(bl, bt, w, bc, &r)) != FSMP_OK) break;
-      ++n_tried;
-      if (r > best) { best = r; bw = w; }
-    }
-    for (int k : {1, 2, 3}) {
-      double r;
-      if (rc != FSMP_OK || (rc = trial(bl, bt, bw, k, &r)) != FSMP_OK) break;
-      ++n_tried;
-      if (r > best) { best = r; bc = k; }
-    }
-    // a team per chain, whatever the number of chains
-    if (rc == FSMP_OK && (lanes0 == 32 || c->pe_lanes_free)) {
-      double r;
-      c->pe_team_always = true;
-      rc = trial(32, tile0, warps0, ctas0, &r);
-      c->pe_team_always = false;
-      if (rc == FSMP_OK) {
-        ++n_tried;
-        if (r > best) { best = r; bteam = true; bl = 32; bt = tile0; bw = warps0; bc = ctas0; }
+  for (int t : tiles) {
+    fsmp_ctx::PeConfig g = best_g;
+    g.tile = t;
+    consider(g, best);
+  }
+  for (int w : {1, 2, 4}) {
+    fsmp_ctx::PeConfig g = best_g;
+    g.warps = w;
+    consider(g, best);
+  }
+  for (int k : {1, 2, 3}) {
+    fsmp_ctx::PeConfig g = best_g;
+    g.ctas = k;
+    consider(g, best);
+  }
+  if (rc == FSMP_OK && best_g.lanes != base.lanes) {
+    rc = in_teams(best_g, &teams);
+    if (rc == FSMP_OK && teams) rc = timed(kTeamAlways, warp0, best_g.lanes, &r_team);
+  }
+  // teams for a number of chains that the rule leaves to a warp per chain: where they are faster on
+  // the sample, the estimate may choose them for any number
+  if (rc == FSMP_OK && !teams && !best_g.team_any) {
+    fsmp_ctx::PeConfig g = best_g;
+    g.team_any = true;
+    if (pe_team_rule(c, best_g, full, &team) == kTeamNever && pe_team_rule(c, g, full, &team) != kTeamNever) {
+      rc = timed(kTeamAlways, warp0, g.lanes, &r);
+      if (rc == FSMP_OK && r > best * kFaster) {
+        best_g.team_any = true;
+        r_team = r;
+        rc = in_teams(best_g, &teams);
       }
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   cudaFree(scratch);
-  if (rc != FSMP_OK) {
-    c->pe_lanes = lanes0; c->pe_tile = tile0; c->pe_warps = warps0; c->p.pe_ctas_per_sm = ctas0;
-    c->pe_tile_free = tfree0;
-    c->pe_team_always = team0;
-    return rc;
+  if (rc != FSMP_OK) return rc;
+  {
+    std::lock_guard<std::mutex> lk(c->launch_mu);
+    c->pe = best_g;
   }
-  c->pe_team_always = bteam;
-  if (best == r0) c->pe_tile_free = tfree0;  // the default launch, with its rules
-  c->pe_lanes = bl; c->pe_tile = bt; c->pe_warps = bw; c->p.pe_ctas_per_sm = bc;
-  if (out) {
-    out->pe_tile = bt; out->chains_per_cta = bteam ? 1 : bw * (32 / bl); out->ctas_per_sm = bc; out->n_tried = n_tried;
-    out->lanes_per_chain = bl;
-    out->best_steps_per_s = best; out->default_steps_per_s = r0;
+  if (out) {  // the launch that the batch will be
+    PeShape s;
+    if (teams) s = team;
+    else pe_shape(c, best_g, B.n_max, b->n_waveforms, &s);
+    out->pe_tile = s.tile;
+    out->chains_per_cta = teams ? 1 : s.warps * (32 / best_g.lanes);
+    out->ctas_per_sm = teams ? 0 : best_g.ctas;
+    out->n_tried = n_tried;
+    out->lanes_per_chain = best_g.lanes;
+    out->best_steps_per_s = teams ? r_team : best; out->default_steps_per_s = r_default;
   }
   return FSMP_OK;
 }
@@ -1333,10 +1388,11 @@ int fsmp_get_info(fsmp_ctx* c, fsmp_info* o) {
   o->R = c->M.R;
   o->L_V = c->M.L_V;
   o->n_smem_max = c->n_smem_max;
-  if (c->p.kernel == FSMP_KERNEL_PE) {  // pe_lanes lanes per chain, pe_warps warps per CTA
+  if (c->p.kernel == FSMP_KERNEL_PE) {
+    const fsmp_ctx::PeConfig g = pe_config(c);
     PeShape s;
-    if (pe_shape(c, c->p.n_max, INT_MAX, &s) == FSMP_OK) {
-      o->threads_per_chain = c->pe_lanes;
+    if (pe_shape(c, g, c->p.n_max, INT_MAX, &s) == FSMP_OK) {
+      o->threads_per_chain = g.lanes;
       o->ctas_per_sm = s.ctas / c->prop.multiProcessorCount;
     }
   } else {

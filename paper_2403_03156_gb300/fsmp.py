@@ -358,7 +358,9 @@ class Context:
     def autotune(self, dev: dict, sample: int = 8192, trial_steps: int = 128, n_steps: int = 0, seed: int = 0,
                  n_max_hint: int = 0) -> dict:
         """fsmp_autotune on device tensors laid out as for run_device: times trial runs of
-        the first `sample` waveforms in candidate launch shapes and keeps the fastest."""
+        the first `sample` waveforms in candidate launch shapes and keeps the fastest. With n_steps,
+        the batch's steps, it knows whether the batch will be launched in teams (else it takes
+        trial_steps for them)."""
         b = _device_batch(dev, n_steps, 0, seed, 0, n_max_hint)
         t = Tune()
         _check(load().fsmp_autotune(self.h, ctypes.byref(b), int(sample), int(trial_steps), ctypes.byref(t)),
