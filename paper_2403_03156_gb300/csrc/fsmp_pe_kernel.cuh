@@ -636,15 +636,14 @@ struct PeStats {
 // eight the batch's loops are twice as long, and wait for instructions too (low occupancy 106 ms
 // against 104, one event 5.97 against 5.22). Up to 32 PEs: beyond, the entries scored for steps
 // that do not count cost what the batch saves. In FP64 mode, where the entries' pair arithmetic is
-// most of a step, that is so from 8 PEs on with 32 lanes and from 12 on with 16 (608 chains of 24 PEs
-// x 150 steps: 6.9 ms with batches up to 32 PEs, 5.8 up to 8; of 8 PEs 5.2 and 4.3; with batches up
-// to 4, 2000 chains of 2 PEs take 6.3 instead of 5.8). 20 000 uneven windows x 2000 steps: 120 -> 110
-// ms, 100 000 low-occupancy chains x 1000: 134 -> 103 ms, 256 FP64 chains x 1000: 13.7 -> 9.8 ms.
+// most of a step, that is so from 12 PEs on (x 300 steps, batches up to 32 PEs and up to 12: 608
+// chains of 24 PEs 15.1 ms and 13.1, of 8 PEs 8.0 and 7.2, 16 of 4 PEs 4.35 and 4.35; with batches up to
+// 8 those 16 take 4.48, with batches up to 4 256 chains of 2 PEs x 1000 13.6 instead of 11.6). 20 000
+// uneven windows x 2000 steps: 120 -> 110 ms, 100 000 low-occupancy chains x 1000: 134 -> 103 ms, 256
+// FP64 chains x 1000: 13.7 -> 9.8 ms.
 constexpr int kSpec = kSub;
 constexpr int kSpecPes = 32;   // most PEs of a chain scored this way (indices in W.ix())
-template <typename T> __host__ __device__ constexpr int spec_pes(int L) {
-  return sizeof(T) == 4 ? kSpecPes : (L == 32 ? 8 : 12);
-}
+template <typename T> __host__ __device__ constexpr int spec_pes() { return sizeof(T) == 4 ? kSpecPes : 12; }
 constexpr int kCounts = 8;     // integer counts of a chain, per subgroup (PeChain::cnt)
 
 // A step's addition to count q: sums over the samples after burn-in of N, N^2, k0 and k0^2, the
@@ -1795,19 +1794,20 @@ __device__ __noinline__ void pe_hist_add(const PeChain<T, BIG, L, MIX> W, uint32
 
 // Resident CTAs per SM the registers are cut for. A chain waits on instruction supply (the code it
 // runs through is larger than a scheduler's instruction cache, which refills at 16 bytes in 2.6
-// cycles), so a warp per chain does as many steps per second with 8 warps per SM as with 16
-// (uneven windows, 20 000 chains x 1000 steps: 58.96 ms against 58.78), each chain at twice the
-// speed: that takes the tail off a launch that has few chains (MCP mixture, 3000 chains: 18.2 ms
-// against 25.7; pile-up, 600 chains: 85.6 against 95.2) and leaves 255 registers. With two chains
-// per warp (L = 16) the half warps wait on each other, and 16 warps are better (30 000
-// low-occupancy chains: 31.5 ms, with 8 warps 42.9).
+// cycles), so cut for 2 CTAs a launch does as many steps per second as cut for 4 (uneven windows,
+// 20 000 chains x 1000 steps: 58.96 ms against 58.78), each chain faster: that takes the tail off a
+// launch that has few chains (MCP mixture, 3000 chains: 18.2 ms against 25.7; pile-up, 600 chains:
+// 85.6 against 95.2). The instances then take, in FP32 mode, 168 registers (dynode: 3 CTAs, 12 warps
+// on an SM), 213 (its pile-up variant) and 180 (mixture: 2 CTAs each), in FP64 mode 168 to 204, and
+// spill nothing. With two chains per warp (L = 16) the half warps wait on each other, and 16 warps are
+// better (30 000 low-occupancy chains: 31.5 ms cut for 4 CTAs, 42.9 for 2), although at 128 registers
+// a step spills (92 bytes stored, 184 loaded); a team's 4 CTAs too (kTeam; pile-up 252 and 520).
 //
-// The mixture's FP32 instance takes 180 registers, so 2 CTAs (8 warps); the dynode one 168 and 3. Its
-// chains of more than 40 PEs gain from the L1 that 2 CTAs leave (608 of 50 PEs x 600 steps: 9.7 ms
-// against 13.6 with 3 CTAs, 5000 of 0.5 to 50 PEs 11.4 against 13.9), but where an SM has enough
-// light chains, 12 warps do more steps than 8: so it comes in both (MORE: 170 registers, 3 CTAs;
-// 16 000 chains: 2 PEs 16.2 -> 13.2 ms, 8 PEs 27.9 -> 23.7, 24 PEs 62.9 -> 58.9, 0.5 to 50 33.6 ->
-// 30.9; n_cap 48, 6000 of 16 PEs 17.2 -> 15.2).
+// The mixture's chains of more than 40 PEs gain from the L1 that 2 CTAs leave (608 of 50 PEs x 600
+// steps: 9.7 ms against 13.6 with 3 CTAs, 5000 of 0.5 to 50 PEs 11.4 against 13.9), but where an SM has
+// enough light chains, 12 warps do more steps than 8: so it comes in both (MORE: 168 registers, 3
+// CTAs; 16 000 chains: 2 PEs 16.2 -> 13.2 ms, 8 PEs 27.9 -> 23.7, 24 PEs 62.9 -> 58.9, 0.5 to 50
+// 33.6 -> 30.9; n_cap 48, 6000 of 16 PEs 17.2 -> 15.2).
 constexpr int pe_min_ctas(int L, int TW, bool MORE) { return L == 16 || TW > 1 ? 4 : (MORE ? 3 : 2); }
 
 template <typename T, bool BIG, int L, bool MIX, int TW = 1, bool MORE = false>
@@ -2081,7 +2081,7 @@ __global__ void __launch_bounds__(kPeMaxThreads, pe_min_ctas(L, TW, MORE))
       bool one = true;         // that step is still to be counted
       unsigned words = 0;
       int last;
-      if (!BIG && N <= spec_pes<T>(L)) {
+      if (!BIG && N <= spec_pes<T>()) {
         // ---------------------------------------------- a batch of steps, one per subgroup
         constexpr int gw = L / kSpec;  // lanes of a subgroup
         const int gi = ln.sl / gw, m = ln.sl % gw;
