@@ -303,12 +303,16 @@ int pe_shape(const fsmp_ctx* c, const fsmp_ctx::PeConfig& g, int n_alloc, int n_
   };
   int per_sm = occupancy(s->smem);
   if (per_sm < 1) return FSMP_ERR_INVALID;
-  // The default tile (40) is 32 where that lets in another CTA that the launch has chains for: the 8
-  // KB more per CTA kept half of the chains out (pile-up model of 1024 samples, 2 CTAs per SM instead
-  // of 1: 6000 chains of 2 PEs x 300 steps 6.4 ms against 9.1, of 35 PEs 32.0 and 31.0; FP64, n_cap
-  // 128, windows of 400: 2000 chains of 15 PEs x 60 steps 4.8 and 5.2).
-  const int resident = per_sm * c->prop.multiProcessorCount * s->warps * (32 / g.lanes);
-  if (g.tile_free && c->pe_c_stride > 0 && s->tile > kTileSmall && n_chains > resident) {
+  // The default tile (40) is 32 where that lets in another CTA that the launch has chains for, more
+  // than 2.5 for each that is resident: the 8 KB more per CTA kept half of the chains out (pile-up
+  // model of 1024 samples, 2 CTAs per SM instead of 1: 4000 chains of 1 to 10 PEs x 300 steps 5.6 ms
+  // against 7.4, of 30 to 200 30.2 and 28.7; 16 lanes, n_cap 128: 12 000 of 0.5 to 30 PEs x 200 9.8 and
+  // 12.7; FP64, n_cap 128: 4000 of 0.5 to 4 PEs x 80 6.0 and 6.6). Launches of fewer chains end with
+  // their longest ones, each faster where fewer share the SM: 16 lanes, 0.5 to 30 PEs x 200, 1300
+  // chains 3.5 and 3.2, 2600 4.4 and 3.6 (but 10 to 30 PEs 4.7 and 5.7), 5000 5.1 and 5.6; pile-up,
+  // 1300 of 30 to 200 PEs x 300 11.4 and 10.4, 2000 15.1 and 15.3; FP64, 700 of 0.5 to 4 1.97 and 1.84.
+  const long long resident = (long long)per_sm * c->prop.multiProcessorCount * s->warps * (32 / g.lanes);
+  if (g.tile_free && c->pe_c_stride > 0 && s->tile > kTileSmall && 2ll * n_chains > 5 * resident) {
     const size_t smem = pe_smem_bytes(c->M, n_alloc, s->warps, g.lanes, kTileSmall, s->form);
     const int more_ctas = occupancy(smem);
     if (more_ctas > per_sm) { per_sm = more_ctas; s->tile = kTileSmall; s->smem = smem; }

@@ -42,3 +42,27 @@ def test_mixture_chains_per_sm(n_cap, n_waveforms, per_sm):
         got.append(d["out"].cpu().numpy())
     for other in got[1:]:
         np.testing.assert_array_equal(got[0], other)
+
+
+@pytest.mark.parametrize("n_waveforms,tile", [(2600, 40), (4000, 32)])
+def test_the_smaller_tile_is_for_launches_of_many_chains(n_waveforms, tile):
+    """16 lanes per chain and n_cap 128: an SM holds one CTA (8 chains) with the tile of 40, two with 32,
+    which a launch takes from 2.5 chains per resident one on (3040 on 152 SMs). The outputs are the
+    same bit for bit."""
+    torch = pytest.importorskip("torch")
+    dev = torch.device("cuda", 0)
+    cfg = workloads.CONFIGS["batched_uneven_100k"]
+    p = dict(cfg["params"], n_cap=128, n_max=512, precision=fsmp.FP32_REFRESH, refresh_every=16, pe_lanes=16, n_streams=1)
+    rng = np.random.Generator(np.random.PCG64(29))
+    b, _ = workloads.simulate(p, np.geomspace(45.0, 0.5, n_waveforms), rng.uniform(30, 40, n_waveforms), rng, "trimmed")
+    got = []
+    for shape in (dict(), dict(pe_tile=32), dict(pe_tile=40)):
+        d = {k: torch.from_numpy(np.ascontiguousarray(b[k])).to(dev) for k in ("samples", "offsets", "lambda0", "t_origin_ns")}
+        d["out"] = torch.zeros(n_waveforms * fsmp.SUMMARY_DTYPE.itemsize, dtype=torch.uint8, device=dev)
+        with gpu_util.context(dict(p, **shape)) as ctx:
+            ctx.run_device(d, n_steps=250, burn_in=20, seed=9, n_max_hint=512)
+            torch.cuda.synchronize(dev)
+            assert ctx.last_launch()["pe_tile"] == shape.get("pe_tile", tile)
+        got.append(d["out"].cpu().numpy())
+    for other in got[1:]:
+        np.testing.assert_array_equal(got[0], other)
