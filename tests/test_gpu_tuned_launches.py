@@ -102,3 +102,28 @@ def test_a_default_shape_that_has_to_shrink_is_timed():
         tune = ctx.autotune(d, sample=200, trial_steps=30, seed=9, n_max_hint=hint)
     print("hint:", hint, "launched:", l, "tuned:", tune)
     assert tune["default_steps_per_s"] > 0 and tune["n_tried"] >= 2
+
+
+def test_a_captured_launch_chooses_its_form_at_each_replay():
+    """1300 chains, beyond those that are all resident as teams: the form is chosen on the device, so
+    a graph captured on light chains runs in teams once its lambda0 are heavy, and the other way round."""
+    torch = pytest.importorskip("torch")
+    p = _params(UNEVEN, n_cap=128)
+    heavy, light = np.geomspace(100, 0.5, 1300), np.full(1300, 2.0)
+    d = _device(UNEVEN, heavy)
+    with gpu_util.context(p) as ctx:
+        want = {}
+        for lam, team in ((heavy, 1), (light, 0)):
+            d["lambda0"].copy_(torch.from_numpy(lam))
+            want[team], launch = _run(ctx, d, 400)
+            assert launch["team"] == team
+        side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            ctx.run_device(d, n_steps=400, burn_in=10, seed=9, n_max_hint=1024, stream=side)
+        for lam, team in ((light, 0), (heavy, 1), (light, 0)):
+            d["lambda0"].copy_(torch.from_numpy(lam))
+            d["out"].zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert ctx.last_launch()["team"] == team
+            np.testing.assert_array_equal(d["out"].cpu().numpy(), want[team])
