@@ -20,8 +20,8 @@
 // a row's address is an offset of the load. The taps travel in the kernel's parameters, a block of
 // them at a 16-byte boundary, and come through the constant cache. Every output adds its taps in the
 // order m = 0, 1, .., L_V - 1, by one FMA each.
-// Arithmetic: 2 (n + L_V) L_V FMAs per iteration, FP32. Bound: issue slots (89 % busy; 61 % of the
-// instructions are FMAs, 12 % source loads), then the FP32 FMA pipe (53 %). 10 000 uneven windows x
+// Arithmetic: 2 (n + L_V) L_V FMAs per iteration, FP32. Bound: issue slots (88 % busy; 61 % of the
+// instructions are FMAs, one in KP as many source loads), then the FP32 FMA pipe (54 %). 10 000 uneven windows x
 // 500 iterations: 6.65 ms, 11.1 ms with 128 outputs a pass, four of them in registers. Packed FMAs
 // (two outputs each) were slower (9.8 ms against 8.3 at that stage): their sources have to be held
 // twice; so were taps from shared memory in place of constants (7.1), and two blocks per turn.
