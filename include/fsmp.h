@@ -351,6 +351,8 @@ typedef struct {
  * trace buffers are not touched (the trials write to scratch). Later results do not depend on
  * the tile, warps, CTAs or teams: a chain's arithmetic is the same in each. They do depend, up to
  * rounding, on the lane count; fix pe_lanes for results reproducible bit for bit.
+ * Windows (n_max_hint, or n_max if 0) that the PE-space kernel does not take leave the context as it
+ * is, with n_tried = 0 and rates of -1.
  * Blocks until the trials finish. Call it with no request in flight on the context. Returns
  * FSMP_OK (out, if not NULL, describes the choice), FSMP_ERR_INVALID (not a PE-space context,
  * bad arguments) or FSMP_ERR_CUDA / FSMP_ERR_NOMEM. */

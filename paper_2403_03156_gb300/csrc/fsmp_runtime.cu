@@ -1218,7 +1218,10 @@ int fsmp_autotune(fsmp_ctx* c, const fsmp_device_batch* b, int sample, int trial
   const fsmp_ctx::PeConfig base = pe_config(c);
   fsmp_ctx::PeConfig best_g = base;
   PeShape warp0, team{};
-  if (pe_shape(c, base, B.n_max, b->n_waveforms, &warp0) != FSMP_OK) FAIL(FSMP_ERR_INVALID, "window too long for the PE-space kernel");
+  if (pe_shape(c, base, B.n_max, b->n_waveforms, &warp0) != FSMP_OK) {  // no launch takes such windows
+    if (out) *out = fsmp_tune{base.tile, base.warps * (32 / base.lanes), base.ctas, 0, -1.0, -1.0, base.lanes};
+    return FSMP_OK;
+  }
   fsmp_summary* scratch = nullptr;
   CK(cudaMalloc(&scratch, sizeof(fsmp_summary) * (size_t)W));
   B.out = scratch;

@@ -68,3 +68,17 @@ def test_tuning_leaves_the_window_limit(precision, n_cap):
     assert not np.any(got.view(fsmp.SUMMARY_DTYPE)["status"] & (fsmp.ST_INVALID | fsmp.ST_BADDET | fsmp.ST_NONFINITE))
     with gpu_util.context(dict(p, pe_lanes=tune["lanes_per_chain"], threads_per_chain=32, pe_tile=8)) as ctx:
         np.testing.assert_array_equal(got, _run(ctx, at_limit, lo))
+
+
+def test_windows_that_no_launch_takes_are_not_tuned_on():
+    pytest.importorskip("torch")
+    p = dict(workloads.CONFIGS["highpileup_20k_1024"]["params"], grid_ns=1.0, precision=fsmp.FP64, n_max=3000, n_streams=1)
+    few = _device(_batch(p, 5, 128, 1))
+    with gpu_util.context(p) as ctx:
+        assert not _accepts(ctx, few, 3000)
+        before = _run(ctx, few, 128), ctx.last_launch()
+        tune = ctx.autotune(few, sample=5, trial_steps=20, seed=3, n_max_hint=3000)
+        assert (tune["n_tried"], tune["best_steps_per_s"], tune["default_steps_per_s"]) == (0, -1.0, -1.0)
+        after = _run(ctx, few, 128), ctx.last_launch()
+    np.testing.assert_array_equal(before[0], after[0])
+    assert before[1] == after[1]
